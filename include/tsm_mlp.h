@@ -18,11 +18,11 @@
  * Gradients use the same layout.
  *
  * Ownership: the model owns its device buffers (parameters, gradients, Adam
- * moments, activations for up to max_batch samples); X (n x D row-major),
- * targets and outputs are caller-owned DEVICE float arrays.  Calls are
- * asynchronous on `stream` except the host<->device parameter copies, which
- * synchronize.  Every reduction over samples runs in sample order, so
- * training is bitwise reproducible.  Errors: INVALID_VALUE for null
+ * moments, partial sums of the gradient); X (n x D row-major), targets and
+ * outputs are caller-owned DEVICE float arrays.  Calls are asynchronous on
+ * `stream` except the host<->device parameter copies, which synchronize.
+ * Every reduction over samples runs in an order fixed by n and the device,
+ * so training is bitwise reproducible.  Errors: INVALID_VALUE for null
  * pointers, n < 1 or n > max_batch, D or H out of range.
  */
 #ifndef TSM_MLP_H
