@@ -11,8 +11,9 @@
  *   TSMTTSM items: a T_M x T_N register tile per thread over the item's rows
  *     (Listing 5, transposed mapping of Fig. 10), lanes reduced in shared
  *     memory, the item's M x N partial written to its own slot; the last item
- *     of an instance to finish sums the instance's slots in item order and
- *     applies alpha/beta (deterministic, no floating-point atomics);
+ *     of a group of consecutive items to finish sums the group's slots in a
+ *     fixed order, and the last group the groups' sums, and applies
+ *     alpha/beta (deterministic, no floating-point atomics);
  *   TSMM items: alpha * C staged in shared memory (Sec. 4.2), TPR threads per
  *     row of B with interleaved results (Fig. 12), two rows per thread per
  *     iteration (Sec. 4.2 unrolling).

@@ -24,6 +24,8 @@ struct Inst {
     double* out;
     double ar, ai, br, bi;
     int64_t part_off;  // doubles: first partial slot of this instance (TSMTTSM)
+    int grp, n_grp;    // items per reduction group, groups
+    int ticket_off;    // tickets of this instance: one, then one per group
 };
 
 struct Item {
@@ -32,10 +34,100 @@ struct Item {
 };
 
 constexpr int kThreads = 256;
-// Work items per persistent CTA the default split aims at.  Items of a few
-// hundred milliseconds (4 per CTA) left SMs idle behind the last large items;
-// 16 per CTA brought the 256-instance mixed batch from 1380 to 1232 ms.
-constexpr double kItemsPerCta = 16.0;
+
+// Sum of the G slots (`stride` doubles apart) of every entry, S threads per
+// entry when there are fewer entries than threads; store(o, v) takes the
+// sum of entry o.  Fixed order: slice s takes slots s, s + S, ..., and the
+// slice sums are combined by a fixed pairwise tree.
+template <int CC, class Store>
+__device__ __forceinline__ void sum_slots(const double* slots, int stride, int G, int MN, double* red,
+                                          const Store& store) {
+    const int t = threadIdx.x;
+    int S = 1;
+    while (S * 2 * MN <= kThreads && S * 2 <= G) S *= 2;
+    for (int base = 0; base < MN * S; base += kThreads) {
+        const int w = base + t;
+        const bool mine = w < MN * S;
+        double v[CC];
+        if (mine) sum_partials<CC>(slots, stride, w / S, G, w % S, S, v);
+        if (S > 1) {
+            // a serial chain over the slices would cost S - 1 FP64 issue
+            // slots in a row
+#pragma unroll
+            for (int c = 0; c < CC; ++c) red[t * CC + c] = mine ? v[c] : 0.0;
+            __syncthreads();
+            for (int h = S >> 1; h >= 1; h >>= 1) {
+                if (mine && (w % S) < h)
+#pragma unroll
+                    for (int c = 0; c < CC; ++c) red[t * CC + c] += red[(t + h) * CC + c];
+                __syncthreads();
+            }
+#pragma unroll
+            for (int c = 0; c < CC; ++c) v[c] = red[t * CC + c];
+            __syncthreads();
+        }
+        if (mine && (w % S) == 0) store(w / S, v);
+    }
+}
+
+// The instance's reduction, called by every thread once its item's partial
+// is in its slot.  The last item of a group of `grp` consecutive items sums
+// the group's slots into its first one; the last group sums those and
+// applies alpha and beta.  One level would leave the whole sum to one CTA
+// (complex 64 x 64 cut into 700 items: 5.7 M adds at 2 a cycle, 1.4 ms on one
+// SM); sqrt(items) groups of sqrt(items) spread it.  Groups and orders are
+// fixed by the plan, so replays repeat bit for bit.
+template <int CC>
+__device__ __noinline__ void reduce_items(const Inst* __restrict__ ip, int idx, double* parts, unsigned* tickets,
+                                          double* red) {
+    __shared__ unsigned s_last;
+    const Inst in = *ip;
+    const int t = threadIdx.x, MN = in.M * in.N, MNc = MN * CC;
+    const int g = idx / in.grp, n_in = min(in.grp, in.n_items - g * in.grp);
+    auto last_of = [&](unsigned* ticket, unsigned n) -> bool {
+        __threadfence();
+        __syncthreads();
+        if (t == 0) {
+            s_last = atomicAdd(ticket, 1u) == n - 1u;
+            if (s_last) *ticket = 0u;  // nobody else takes it before the next launch
+        }
+        __syncthreads();
+        const bool last = s_last != 0u;
+        if (last) __threadfence();
+        return last;
+    };
+    auto finish = [&](int o, const double* v) {
+        const int m = o / in.N, n = o - m * in.N;
+        double* out = in.out + ((int64_t)m * in.ldo + n) * CC;
+        if (CC == 1) {
+            double r = in.ar * v[0];
+            if (!in.beta_zero) r = fma(in.br, out[0], r);
+            out[0] = r;
+        } else {
+            double rr = in.ar * v[0] - in.ai * v[CC - 1];
+            double ri = in.ar * v[CC - 1] + in.ai * v[0];
+            if (!in.beta_zero) {
+                const double orr = out[0], oi = out[CC - 1];
+                rr += in.br * orr - in.bi * oi;
+                ri += in.br * oi + in.bi * orr;
+            }
+            out[0] = rr;
+            out[CC - 1] = ri;
+        }
+    };
+    if (!last_of(&tickets[in.ticket_off + 1 + g], (unsigned)n_in)) return;
+    double* slots = parts + in.part_off + (int64_t)g * in.grp * MNc;
+    if (in.n_grp == 1) {
+        sum_slots<CC>(slots, MNc, n_in, MN, red, finish);
+        return;
+    }
+    sum_slots<CC>(slots, MNc, n_in, MN, red, [&](int o, const double* v) {
+#pragma unroll
+        for (int c = 0; c < CC; ++c) slots[o * CC + c] = v[c];
+    });
+    if (!last_of(&tickets[in.ticket_off], (unsigned)in.n_grp)) return;
+    sum_slots<CC>(parts + in.part_off, in.grp * MNc, in.n_grp, MN, red, finish);
+}
 
 // ----------------------------------------------------------- TSMTTSM item
 
@@ -66,7 +158,6 @@ __device__ __noinline__ void tsmttsm_item(const Inst* __restrict__ ip, const Ite
                                           unsigned* tickets, double* red) {
     const Inst in = *ip;
     constexpr int CC = CPLX ? 2 : 1;
-    __shared__ unsigned s_last;
     const int M = in.M, N = in.N;
     const int PM = (M + TM - 1) / TM, PN = (N + TN - 1) / TN, P = PM * PN;
     const int L = kThreads / P;
@@ -155,58 +246,7 @@ __device__ __noinline__ void tsmttsm_item(const Inst* __restrict__ ip, const Ite
                 }
                 __syncthreads();
             }
-    __threadfence();
-    __syncthreads();
-    if (t == 0) s_last = (atomicAdd(&tickets[it.inst], 1u) == (unsigned)in.n_items - 1u);
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    const double* slots = parts + in.part_off;
-    const int MN = M * N, G = in.n_items;
-    int S = 1;
-    while (S * 2 * MN <= kThreads && S * 2 <= G) S *= 2;
-    for (int base = 0; base < MN * S; base += kThreads) {
-        const int w = base + t;
-        const bool mine = w < MN * S;
-        double v[CC];
-        if (mine) sum_partials<CC>(slots, MNc, w / S, G, w % S, S, v);
-        if (S > 1) {
-            // fixed pairwise tree over the S slice sums of one entry (a
-            // serial chain would cost S - 1 FP64 issue slots in a row)
-#pragma unroll
-            for (int c = 0; c < CC; ++c) red[t * CC + c] = mine ? v[c] : 0.0;
-            __syncthreads();
-            for (int h = S >> 1; h >= 1; h >>= 1) {
-                if (mine && (w % S) < h)
-#pragma unroll
-                    for (int c = 0; c < CC; ++c) red[t * CC + c] += red[(t + h) * CC + c];
-                __syncthreads();
-            }
-#pragma unroll
-            for (int c = 0; c < CC; ++c) v[c] = red[t * CC + c];
-            __syncthreads();
-        }
-        if (!mine || (w % S) != 0) continue;
-        const int o = w / S, m = o / N, n = o - m * N;
-        double* out = in.out + ((int64_t)m * in.ldo + n) * CC;
-        if (!CPLX) {
-            double r = in.ar * v[0];
-            if (!in.beta_zero) r = fma(in.br, out[0], r);
-            out[0] = r;
-        } else {
-            double rr = in.ar * v[0] - in.ai * v[CC - 1];
-            double ri = in.ar * v[CC - 1] + in.ai * v[0];
-            if (!in.beta_zero) {
-                const double orr = out[0], oi = out[CC - 1];
-                rr += in.br * orr - in.bi * oi;
-                ri += in.br * oi + in.bi * orr;
-            }
-            out[0] = rr;
-            out[CC - 1] = ri;
-        }
-    }
-    __syncthreads();
-    if (t == 0) tickets[it.inst] = 0u;
+    reduce_items<CC>(ip, it.idx, parts, tickets, red);
 }
 
 // -------------------------------------------------------------- TSMM item
@@ -559,6 +599,58 @@ int default_tile(int M, int N, int cplx) {
     return best;
 }
 
+// What a row of an instance costs, in cycles of one SM: the FP64 issue slots
+// it takes (2 a cycle, idle lanes and padded tile entries included) or its
+// bytes at an SM's share of the memory rate (21 a cycle), whichever is more.
+// `floor`: the least an item should cost, so that staging C, or reducing an
+// M x N partial twice, stays near a tenth of it (half of it, or a quarter,
+// measured the same to 10 % slower on batches of 4 to 64 small products).  `quantum`: rows the CTA
+// takes per pass.
+struct RowCost {
+    double row, floor;
+    int64_t quantum;
+};
+
+RowCost row_cost(const Inst& in) {
+    const int c = in.cplx ? 2 : 1, fma = in.cplx ? 4 : 1;
+    const double MNc = (double)in.M * in.N * c;
+    double slots;
+    int lanes, unroll;
+    if (in.kind == TSM_KIND_TSMTTSM) {
+        int tm, tn;
+        code_tile(in.code, in.cplx, &tm, &tn);
+        const int P = ((in.M + tm - 1) / tm) * ((in.N + tn - 1) / tn);
+        lanes = kThreads / P;
+        unroll = tm * tn >= 14 ? 1 : (tm * tn == 1 ? 4 : 2);
+        slots = (double)((P * lanes + 31) / 32 * 32) * tm * tn * fma / lanes;
+    } else {
+        const int tpr = in.code == 4 ? in.tpr : (in.code == 3 ? 16 : (in.code == 1 && !in.cplx ? 4 : 8));
+        lanes = kThreads / tpr;
+        unroll = 2;
+        slots = (double)((lanes * tpr + 31) / 32 * 32) * ((in.N + tpr - 1) / tpr) * in.M * fma / lanes;
+    }
+    RowCost r;
+    r.row = std::max(slots / 2.0, 8.0 * c * (in.M + in.N) / 21.0);
+    r.floor = 20000.0 + (in.kind == TSM_KIND_TSMTTSM ? 12.0 : 8.0) * MNc;
+    r.quantum = (int64_t)lanes * unroll;
+    return r;
+}
+
+// How the default split cuts an instance: three quarters of its rows into
+// items of an eighth of a CTA's share of the whole batch, then smaller ones.
+// Claimed largest first, the small ones fill the end, so the CTAs finish
+// within about a hundredth of the batch of one another.  Measured, with the
+// first tier at 1/4, 1/8, 1/16 (the others in the same ratio): 1254, 1216,
+// 1213 ms for 256 products of 2^16 .. 2^22 rows, 17.5, 16.8, 17.0 ms for 32
+// of 2^14 .. 2^18, 0.95, 0.95, 1.06 ms for 64 of 2^10 .. 2^12.  Equal items of
+// at least 4096 rows, the split before this one, took 1231, 29.4 and 22.4 ms:
+// a 4096-row item of a complex 64 x 64 product alone takes 16 ms on one CTA.
+struct Tier {
+    double part, share;
+};
+constexpr int kTiers = 3;
+constexpr Tier kTier[kTiers] = {{0.75, 1.0 / 8}, {0.2, 1.0 / 32}, {0.05, 1.0 / 128}};
+
 }  // namespace batched
 }  // namespace tsm
 
@@ -630,15 +722,9 @@ tsm_status tsm_batched_create(const tsm_batch_desc* d, int count, tsm_batch** ou
 
     // instance table and work items
     std::vector<Inst> inst(count);
-    double total = 0.0;
-    std::vector<double> work(count);
-    for (int i = 0; i < count; ++i) {
-        const int c = d[i].dtype == TSM_C64 ? 2 : 1;
-        work[i] = (double)d[i].K * d[i].M * d[i].N * c * c + 1.0;
-        total += work[i];
-    }
     std::vector<Item> items;
-    int64_t part_doubles = 0;
+    std::vector<RowCost> cost(count);
+    double total = 0.0;
     for (int i = 0; i < count; ++i) {
         const tsm_batch_desc& x = d[i];
         Inst& in = inst[i];
@@ -677,42 +763,54 @@ tsm_status tsm_batched_create(const tsm_batch_desc* d, int count, tsm_batch** ou
             int npt = 1;
             rt_tsmm_tpr(x.N, 4, &in.tpr, &npt);
         }
-        int64_t rows;
-        const int lg = (x.config >> 8) & 0xFF;
+        cost[i] = row_cost(in);
+        total += (double)x.K * cost[i].row;
+    }
+    int64_t part_doubles = 0;
+    int n_tickets = 0;
+    for (int i = 0; i < count; ++i) {
+        Inst& in = inst[i];
+        const int first = (int)items.size();
+        const int lg = (d[i].config >> 8) & 0xFF;
+        auto cut = [&](int64_t from, int64_t to, int64_t rows) {
+            do {
+                Item it;
+                it.inst = i;
+                it.idx = (int)items.size() - first;
+                it.r0 = from;
+                it.r1 = std::min(to, from + rows);
+                items.push_back(it);
+                from = it.r1;
+            } while (from < to);
+        };
         if (lg >= 10 && lg <= 22) {
-            rows = (int64_t)1 << lg;
+            cut(0, in.K, (int64_t)1 << lg);
         } else {
-            // about kItemsPerCta items per CTA over the whole batch, each
-            // instance cut in proportion to its work; rows per item the
-            // nearest power of two (at least 4096), so an instance ends in a
-            // shorter ragged item and the largest-first order finishes on
-            // small items
-            const double share = work[i] / total * ctas * kItemsPerCta;
-            const double n = std::max(1.0, std::floor(share));
-            const int l = (int)std::lround(std::log2(std::max((double)x.K / n, 1.0)));
-            rows = (int64_t)1 << std::min(22, std::max(12, l));
+            int64_t from = 0;
+            for (int tier = 0; tier < kTiers; ++tier) {
+                const double want = std::max(kTier[tier].share * total / ctas, cost[i].floor);
+                const double rows = std::min(want / cost[i].row, (double)in.K + 1.0);
+                const int64_t q = cost[i].quantum;
+                const int64_t r = std::max<int64_t>(1, (int64_t)std::ceil(rows / q)) * q;
+                int64_t to = tier == kTiers - 1 ? in.K : from + (int64_t)(kTier[tier].part * (double)in.K) / r * r;
+                if (in.K - to < r) to = in.K;  // no crumb for the next tier
+                if (to > from || (in.K == 0 && tier == 0)) cut(from, to, r);
+                from = to;
+            }
         }
-        const int64_t K = std::max<int64_t>(x.K, 1);
-        const int n_items = (int)((K + rows - 1) / rows);
-        in.n_items = n_items;
+        in.n_items = (int)items.size() - first;
         in.part_off = part_doubles;
-        if (x.kind == TSM_KIND_TSMTTSM) part_doubles += (int64_t)n_items * x.M * x.N * (in.cplx ? 2 : 1);
-        for (int j = 0; j < n_items; ++j) {
-            Item it;
-            it.inst = i;
-            it.idx = j;
-            it.r0 = std::min<int64_t>((int64_t)j * rows, x.K);
-            it.r1 = std::min<int64_t>((int64_t)(j + 1) * rows, x.K);
-            items.push_back(it);
+        in.grp = in.n_items <= 16 ? in.n_items : (int)std::ceil(std::sqrt((double)in.n_items));
+        in.n_grp = (in.n_items + in.grp - 1) / in.grp;
+        in.ticket_off = n_tickets;
+        if (in.kind == TSM_KIND_TSMTTSM) {
+            part_doubles += (int64_t)in.n_items * in.M * in.N * (in.cplx ? 2 : 1);
+            n_tickets += 1 + in.n_grp;
         }
     }
     // largest items first (list scheduling over the persistent CTAs)
     std::stable_sort(items.begin(), items.end(), [&](const Item& a, const Item& b) {
-        const Inst& ia = inst[a.inst];
-        const Inst& ib = inst[b.inst];
-        const double ca = (double)(a.r1 - a.r0 + 1) * ia.M * ia.N * (ia.cplx ? 4 : 1);
-        const double cb = (double)(b.r1 - b.r0 + 1) * ib.M * ib.N * (ib.cplx ? 4 : 1);
-        return ca > cb;
+        return (double)(a.r1 - a.r0 + 1) * cost[a.inst].row > (double)(b.r1 - b.r0 + 1) * cost[b.inst].row;
     });
 
     tsm_batch* b = (tsm_batch*)calloc(1, sizeof(tsm_batch));
@@ -724,7 +822,7 @@ tsm_status tsm_batched_create(const tsm_batch_desc* d, int count, tsm_batch** ou
     bool ok = cudaMalloc(&b->d_inst, sizeof(Inst) * count) == cudaSuccess &&
               cudaMalloc(&b->d_items, sizeof(Item) * items.size()) == cudaSuccess &&
               cudaMalloc(&b->d_counter, sizeof(unsigned)) == cudaSuccess &&
-              cudaMalloc(&b->d_tickets, sizeof(unsigned) * count) == cudaSuccess &&
+              cudaMalloc(&b->d_tickets, sizeof(unsigned) * std::max(n_tickets, 1)) == cudaSuccess &&
               cudaMalloc(&b->d_parts, sizeof(double) * std::max<int64_t>(part_doubles, 1)) == cudaSuccess;
     if (!ok) {
         tsm_batched_destroy(b);
@@ -732,7 +830,7 @@ tsm_status tsm_batched_create(const tsm_batch_desc* d, int count, tsm_batch** ou
     }
     if (cudaMemcpy(b->d_inst, inst.data(), sizeof(Inst) * count, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(b->d_items, items.data(), sizeof(Item) * items.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemset(b->d_tickets, 0, sizeof(unsigned) * count) != cudaSuccess) {
+        cudaMemset(b->d_tickets, 0, sizeof(unsigned) * std::max(n_tickets, 1)) != cudaSuccess) {
         tsm_batched_destroy(b);
         return TSM_ERR_LAUNCH;
     }
