@@ -21,34 +21,55 @@ __all__ = ["tsmttsm", "tsmm", "gs_step", "fill_random", "variants", "variant_sha
 _OPS = {"T": OP_T, "C": OP_C, "N": OP_N, OP_T: OP_T, OP_C: OP_C, OP_N: OP_N}
 
 
+# The helpers below run several times per call.  A product of a few thousand
+# rows takes the GPU about 10 us; marshalling took the host 9 us of 15.8 in
+# all (3 of them the torch.cuda.Stream object of the current stream), which
+# set the time of every short call.
+
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def _dtype_code(t):
     torch = _torch()
-    if t.dtype == torch.float64:
+    dt = t.dtype
+    if dt is torch.float64:
         return R64
-    if t.dtype == torch.complex128:
+    if dt is torch.complex128:
         return C64
-    raise TypeError("tensors must be float64 or complex128, got %s" % t.dtype)
+    raise TypeError("tensors must be float64 or complex128, got %s" % dt)
 
 
 def _ld(t, name):
-    if t.dim() != 2:
+    shape = t.shape
+    if len(shape) != 2:
         raise ValueError("%s must be 2-D" % name)
-    if t.shape[1] > 1 and t.stride(1) != 1:
+    rows, cols = t.stride()
+    width = shape[1]
+    if width > 1 and cols != 1:
         raise ValueError("%s must be row-major (stride(1) == 1)" % name)
     if not t.is_cuda:
         raise ValueError("%s must be a CUDA tensor" % name)
-    return max(int(t.stride(0)), int(t.shape[1]))
+    return rows if rows > width else width
 
 
 def _stream(stream):
-    torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    """Address of a stream, the current one of the current device for None
+    (asked for as such, without a torch.cuda.Stream object around it)."""
+    if stream is None:
+        torch = _torch()
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is not None and torch.cuda.is_initialized():
+            return raw(torch._C._cuda_getDevice())
+        stream = torch.cuda.current_stream()
+    return stream.cuda_stream
 
 
 def tsmttsm(A, B, C=None, alpha=1.0, beta=0.0, op="T", stream=None, variant=-1, grid=0):
@@ -63,9 +84,9 @@ def tsmttsm(A, B, C=None, alpha=1.0, beta=0.0, op="T", stream=None, variant=-1, 
         C = torch.zeros((M, N), dtype=A.dtype, device=A.device)
         beta = 0.0
     cplx = dt == C64
-    call("tsm_tsmttsm_ex", _OPS[op], dt, M, N, K, scalar(alpha, cplx), ctypes.c_void_p(A.data_ptr()),
-         _ld(A, "A"), ctypes.c_void_p(B.data_ptr()), _ld(B, "B"), scalar(beta, cplx),
-         ctypes.c_void_p(C.data_ptr()), _ld(C, "C"), int(variant), int(grid), _stream(stream))
+    call("tsm_tsmttsm_ex", _OPS[op], dt, M, N, K, scalar(alpha, cplx), A.data_ptr(),
+         _ld(A, "A"), B.data_ptr(), _ld(B, "B"), scalar(beta, cplx),
+         C.data_ptr(), _ld(C, "C"), int(variant), int(grid), _stream(stream))
     return C
 
 
@@ -81,8 +102,8 @@ def tsmm(A, Cm, B=None, alpha=1.0, beta=0.0, stream=None, variant=-1, grid=0):
         B = torch.empty((K, N), dtype=A.dtype, device=A.device)
         beta = 0.0
     cplx = dt == C64
-    call("tsm_tsmm_ex", OP_N, dt, M, N, K, scalar(alpha, cplx), ctypes.c_void_p(A.data_ptr()), _ld(A, "A"),
-         ctypes.c_void_p(Cm.data_ptr()), _ld(Cm, "C"), scalar(beta, cplx), ctypes.c_void_p(B.data_ptr()),
+    call("tsm_tsmm_ex", OP_N, dt, M, N, K, scalar(alpha, cplx), A.data_ptr(), _ld(A, "A"),
+         Cm.data_ptr(), _ld(Cm, "C"), scalar(beta, cplx), B.data_ptr(),
          _ld(B, "B"), int(variant), int(grid), _stream(stream))
     return B
 
@@ -104,8 +125,8 @@ def gs_step(A, B, C=None, stream=None, mode="auto"):
         C = torch.empty((M, N), dtype=A.dtype, device=A.device)
     elif C.shape != (M, N) or _dtype_code(C) != dt:
         raise ValueError("C must be M x N with A's dtype")
-    call("tsm_gs_step_ex", dt, M, N, K, ctypes.c_void_p(A.data_ptr()), _ld(A, "A"), ctypes.c_void_p(B.data_ptr()),
-         _ld(B, "B"), ctypes.c_void_p(C.data_ptr()), _ld(C, "C"), GS_MODES[mode], _stream(stream))
+    call("tsm_gs_step_ex", dt, M, N, K, A.data_ptr(), _ld(A, "A"), B.data_ptr(),
+         _ld(B, "B"), C.data_ptr(), _ld(C, "C"), GS_MODES[mode], _stream(stream))
     return C
 
 

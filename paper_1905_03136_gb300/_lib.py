@@ -93,6 +93,8 @@ def extend_signatures(extra):
 def load():
     """Loads libtsm.so (raises if it is missing: there is no fallback)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
@@ -127,10 +129,14 @@ def check(status, where):
     return status
 
 
+_Scalar = ctypes.c_double * 2
+
+
 def scalar(x, cplx):
+    if type(x) is float:
+        return _Scalar(x, 0.0)
     z = complex(x)
-    arr = (ctypes.c_double * 2)(z.real, z.imag if cplx else 0.0)
-    return arr
+    return _Scalar(z.real, z.imag if cplx else 0.0)
 
 
 def call(name, *args):

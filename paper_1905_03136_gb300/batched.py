@@ -57,9 +57,8 @@ class Batch:
         self.h = h
 
     def _stream(self, stream):
-        import torch
-        s = stream if stream is not None else torch.cuda.current_stream()
-        return ctypes.c_void_p(s.cuda_stream)
+        from . import _stream
+        return _stream(stream)
 
     def run(self, stream=None):
         _lib.call("tsm_batched_run", self.h, self._stream(stream))

@@ -24,9 +24,8 @@ _lib.extend_signatures({
 
 
 def _stream(stream):
-    import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    from . import _stream as address
+    return address(stream)
 
 
 class Mlp:

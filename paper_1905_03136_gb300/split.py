@@ -47,9 +47,9 @@ def tsmttsm_split(A, B, C=None, alpha=1.0, beta=0.0, op="T", stream=None, slices
         C = torch.zeros((M, N), dtype=A.dtype, device=A.device)
         beta = 0.0
     cplx = dt == 1
-    _lib.call("tsm_tsmttsm_split_ex", _OPS[op], dt, M, N, K, scalar(alpha, cplx), ctypes.c_void_p(A.data_ptr()),
-              _ld(A, "A"), ctypes.c_void_p(B.data_ptr()), _ld(B, "B"), scalar(beta, cplx),
-              ctypes.c_void_p(C.data_ptr()), _ld(C, "C"), int(kind), int(slices), _stream(stream))
+    _lib.call("tsm_tsmttsm_split_ex", _OPS[op], dt, M, N, K, scalar(alpha, cplx), A.data_ptr(),
+              _ld(A, "A"), B.data_ptr(), _ld(B, "B"), scalar(beta, cplx),
+              C.data_ptr(), _ld(C, "C"), int(kind), int(slices), _stream(stream))
     return C
 
 
