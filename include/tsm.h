@@ -166,7 +166,8 @@ int tsm_variant_supports(tsm_kind kind, int index, tsm_dtype dtype, int M, int N
 /* Kernel launches one TSMTTSM call of shape (dtype, M, N) makes with `grid`
  * CTAs: 1, or 2 when the CTA partials (grid * M * N doubles, twice that for
  * complex) are many enough that a separate final kernel sums them (Sec. 3.2
- * reduction, second pass).  -1 for a shape outside [1, 64] or grid < 1. */
+ * reduction, second pass).  The row variants (tsmttsm_*_row, which short
+ * products take) always make 2.  -1 for a shape outside [1, 64] or grid < 1. */
 int tsm_tsmttsm_kernels_per_call(tsm_dtype dtype, int M, int N, int grid);
 
 /*

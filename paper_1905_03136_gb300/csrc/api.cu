@@ -115,25 +115,24 @@ std::mutex g_occ_mutex;
 std::map<std::pair<int, OccKey>, int> g_occ;  // (device, kernel shape) -> resident CTAs per SM
 }  // namespace
 
+int resident_ctas(const void* kernel, int block, size_t smem) {
+    const auto key = std::make_pair(device_info().device, OccKey{kernel, block, smem});
+    std::lock_guard<std::mutex> lock(g_occ_mutex);
+    auto it = g_occ.find(key);
+    if (it != g_occ.end()) return it->second;
+    int occ = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, block, smem) != cudaSuccess) {
+        cudaGetLastError();
+        occ = 0;
+    }
+    g_occ[key] = occ;
+    return occ;
+}
+
 bool pdl_allowed(const void* kernel, int grid, int block, size_t smem) {
     if (!pdl_enabled()) return false;
-    const DeviceInfo& di = device_info();
-    const auto key = std::make_pair(di.device, OccKey{kernel, block, smem});
-    int occ = 0;
-    {
-        std::lock_guard<std::mutex> lock(g_occ_mutex);
-        auto it = g_occ.find(key);
-        if (it != g_occ.end()) {
-            occ = it->second;
-        } else {
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, block, smem) != cudaSuccess) {
-                cudaGetLastError();
-                occ = 0;
-            }
-            g_occ[key] = occ;
-        }
-    }
-    return occ > 0 && (int64_t)grid >= (int64_t)occ * di.sm_count;
+    const int occ = resident_ctas(kernel, block, smem);
+    return occ > 0 && (int64_t)grid >= (int64_t)occ * device_info().sm_count;
 }
 
 Range operand_range(const void* p, int64_t rows, int64_t ld, int cols, int cplx) {
@@ -227,6 +226,7 @@ struct Registry {
         register_generated_variants(tsmttsm, tsmm);
         register_rt_variants(tsmttsm, tsmm);
         register_narrow_variants(tsmttsm, tsmm);
+        register_row_variants(tsmttsm);
     }
 };
 
@@ -245,6 +245,7 @@ static bool variant_supports(const Variant& v, int dtype, int M, int N) {
     if (v.info.dtype != dtype) return false;
     if (v.info.fixed_m && v.info.fixed_m != M) return false;
     if (v.info.fixed_n && v.info.fixed_n != N) return false;
+    if (v.supports) return M >= 1 && N >= 1 && M <= 64 && N <= 64 && v.supports(M, N);
     if (v.info.runtime_tile) return M >= 1 && N >= 1 && M <= 64 && N <= 64;  // a tile always exists
     if (v.info.kind == TSM_KIND_TSMTTSM) {
         const int P = ((M + v.info.tile_m - 1) / v.info.tile_m) * ((N + v.info.tile_n - 1) / v.info.tile_n);
@@ -274,7 +275,7 @@ static int heuristic_variant(tsm_kind kind, int dtype, int M, int N) {
         int best_area = 0, best_u = 0;
         for (size_t i = 0; i < t.size(); ++i) {
             const tsm_variant_info& f = t[i].info;
-            if (f.generated || !variant_supports(t[i], dtype, M, N)) continue;
+            if (f.generated || f.runtime_tile || !variant_supports(t[i], dtype, M, N)) continue;
             const int pm = (M + f.tile_m - 1) / f.tile_m, pn = (N + f.tile_n - 1) / f.tile_n;
             const double waste = (double)(pm * f.tile_m) * (pn * f.tile_n) / ((double)M * N);
             const int area = f.tile_m * f.tile_n;
@@ -318,26 +319,85 @@ static int heuristic_variant(tsm_kind kind, int dtype, int M, int N) {
     return -1;
 }
 
-static int default_grid(const Variant& v, int M, int N) {
+static int default_grid(const Variant& v, int M, int N, int64_t K) {
+    if (v.grid) return v.grid(M, N, K);
     const int occ = v.occupancy ? v.occupancy(M, N) : 1;
     return device_info().sm_count * (occ > 0 ? occ : 1);
+}
+
+static int find_named(tsm_kind kind, const char* name) {
+    const std::vector<Variant>& t = *table(kind);
+    for (size_t i = 0; i < t.size(); ++i)
+        if (strcmp(t[i].info.name, name) == 0) return (int)i;
+    return -1;
+}
+
+// FP64 slots per useful FMA of a TSMTTSM variant: padding of its tile past M
+// and N times the idle lanes of its CTA's last warp.
+static double tile_slots(const tsm_variant_info& f, int M, int N) {
+    const int P = ((M + f.tile_m - 1) / f.tile_m) * ((N + f.tile_n - 1) / f.tile_n);
+    const int L = P <= f.block ? f.block / P : 1;
+    return (double)((P * L + 31) / 32 * 32) * f.tile_m * f.tile_n / ((double)L * M * N);
+}
+
+// Whether the row kernel (kernels_row.cu) runs a product below 2^21 rows
+// instead of `other` (the nearest tuned entry's variant, or the heuristic's).
+// Measured, us a call, other / row kernel:
+//   up to 10^8 FMAs, whose time is mostly the other kernels' reduction tails:
+//     real 8 x 8, 16000 rows 16.4 / 10.2; real 6 x 6, 50000 rows 48 / 9.1; complex
+//     8 x 8, 10^5 rows 53 / 45; real 25 x 25, 60000 rows 96 / 71; real 64 x 64,
+//     16000 rows 131 / 116.  At 2.5 10^8 they meet (complex 32 x 32, 60000 rows
+//     406 / 420, real 25 x 25, 250000 rows 286 / 289).
+//   fewer than 64 FMAs a row on a kernel without padding are bound by memory
+//     from about 5 10^6 FMAs or 16 MB on, where the vector-streaming kernels
+//     and the 1 x 1 tile win: real 4 x 4, 250000 rows 16.4 / 13.4, 900000 rows
+//     33.8 / 33.5, 1.9 10^6 rows 64 / 78; complex 1 x 12, 250000 rows 33.5 /
+//     37.4; real 2 x 2, 10^6 rows 26.6 / 33.8 inside a Gram-Schmidt step.
+//   the shortest products on the vector-streaming kernels (up to 5 10^5 FMAs)
+//     take 8 to 10 us of GPU time in one launch; the row kernel's 6 to 9 us in
+//     two launches are then hidden by the host's 10.
+//   longer products without a tuned entry, by the slots their tiles waste:
+//     real 37 x 53, 300007 rows 1119 / 999 (1.14 against 1.03); complex 17 x 33,
+//     200000 rows 880 / 788; real 9 x 41, 10^6 rows 671 / 690 (1.04, 1.03: stays).
+static bool row_preferred(const tsm_variant_info& other, bool tuned, int dtype, int M, int N, int64_t K) {
+    const double slots = row_slots(M, N, dtype == TSM_C64);
+    if (slots <= 0.0 || K >= ((int64_t)1 << 21)) return false;
+    const double per_row = (double)M * N * (dtype == TSM_C64 ? 4 : 1), fma = per_row * (double)K;
+    const bool narrow = strstr(other.name, "narrow") != nullptr;
+    const double waste = narrow ? 1.0 : tile_slots(other, M, N);
+    const bool small_tile = narrow || (!other.generated && other.tile_m * other.tile_n <= 4);
+    if (narrow && fma < 5e5) return false;
+    if (per_row < 64.0 && small_tile && waste < 1.3)
+        return fma <= 5e6 && 8.0 * (dtype == TSM_C64 ? 2 : 1) * (M + N) * (double)K <= 1.7e7;
+    if (short_product(M, N, K, dtype == TSM_C64)) return true;
+    return !tuned && slots * 1.05 < waste;
 }
 
 tsm_status choose(tsm_kind kind, int dtype, int M, int N, int64_t K, int* variant, int* grid) {
     const std::vector<Variant>* t = table(kind);
     if (!t) return TSM_ERR_INVALID_VALUE;
-    int v = -1, g = 0;
+    int v = -1, g = 0, distance = -1;
     auto looked_up = [&](tsm_kind k) {
-        return tune_lookup(k, dtype, M, N, K, &v, &g) == TSM_OK && v >= 0 && v < (int)t->size() &&
+        return tune_lookup(k, dtype, M, N, K, &v, &g, &distance) == TSM_OK && v >= 0 && v < (int)t->size() &&
                variant_supports((*t)[v], dtype, M, N);
     };
     // TSMM with beta != 0: its own entry first, else the beta = 0 one
     if (!looked_up(kind) && !(kind == TSM_KIND_TSMM_BETA && looked_up(TSM_KIND_TSMM))) {
         v = heuristic_variant(kind == TSM_KIND_TSMM_BETA ? TSM_KIND_TSMM : kind, dtype, M, N);
         g = 0;
+        distance = -1;
     }
     if (v < 0) return TSM_ERR_NOT_SUPPORTED;
-    if (g <= 0) g = default_grid((*t)[v], M, N);
+    // an entry tuned for this very bucket of K stands
+    if (kind == TSM_KIND_TSMTTSM && distance != 0 && row_preferred((*t)[v].info, distance > 0, dtype, M, N, K)) {
+        static const int row[2] = {find_named(TSM_KIND_TSMTTSM, "tsmttsm_r64_row"),
+                                   find_named(TSM_KIND_TSMTTSM, "tsmttsm_c64_row")};
+        if (row[dtype == TSM_C64] >= 0) {
+            v = row[dtype == TSM_C64];
+            g = 0;
+        }
+    }
+    if (g <= 0) g = default_grid((*t)[v], M, N, K);
     *variant = v;
     *grid = g;
     return TSM_OK;
@@ -402,7 +462,7 @@ tsm_status run_tsmttsm(tsm_op opA, tsm_dtype dtype, int M, int N, int64_t K, con
     }
     if (!supports(TSM_KIND_TSMTTSM, v, dtype, M, N)) return TSM_ERR_NOT_SUPPORTED;
     const Variant& var = *variant_at(TSM_KIND_TSMTTSM, v);
-    if (g <= 0) g = default_grid(var, M, N);
+    if (g <= 0) g = default_grid(var, M, N, K);
     if (g > 65535) g = 65535;
 
     Workspace* ws = nullptr;
@@ -427,7 +487,7 @@ tsm_status run_tsmttsm(tsm_op opA, tsm_dtype dtype, int M, int N, int64_t K, con
     a.conj = (cplx && opA == TSM_OP_C) ? 1 : 0;
     a.ws = ws->partials;
     a.ticket = ws->tickets;
-    a.final_pass = tsm_tsmttsm_kernels_per_call(dtype, M, N, g) == 2 ? 1 : 0;
+    a.final_pass = var.final_pass || tsm_tsmttsm_kernels_per_call(dtype, M, N, g) == 2 ? 1 : 0;
     const Range in[2] = {operand_range(A, K, lda, M, cplx), operand_range(B, K, ldb, N, cplx)};
     std::lock_guard<std::mutex> lock(pdl_mutex());
     a.early = pdl_early(stream, in, 2);
@@ -467,7 +527,7 @@ tsm_status run_tsmm(tsm_op opC, tsm_dtype dtype, int M, int N, int64_t K, const 
     }
     if (!supports(TSM_KIND_TSMM, v, dtype, M, N)) return TSM_ERR_NOT_SUPPORTED;
     const Variant& var = *variant_at(TSM_KIND_TSMM, v);
-    if (g <= 0) g = default_grid(var, M, N);
+    if (g <= 0) g = default_grid(var, M, N, K);
     if (g > 65535) g = 65535;
     TsmmArgs a;
     a.M = M;

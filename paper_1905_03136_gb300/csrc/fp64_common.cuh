@@ -30,6 +30,37 @@ __device__ __forceinline__ void sum_partials(const double* ws, int MNc, int o, i
                  ((acc[c][4] + acc[c][5]) + (acc[c][6] + acc[c][7]));
 }
 
+// The same sums with the last partials of a slice loaded as one more batch
+// instead of one at a time (each alone would wait for L2 in turn: at 304
+// partials over 32 lanes, two of 10 loads).  For the kernels that only
+// reduce, or whose reduction sets their time.
+template <int CC>
+__device__ __forceinline__ void sum_partials_batched(const double* ws, int stride, int o, int G, int s, int S,
+                                                     double* out) {
+    double acc[CC][8];
+#pragma unroll
+    for (int c = 0; c < CC; ++c)
+#pragma unroll
+        for (int r = 0; r < 8; ++r) acc[c][r] = 0.0;
+    for (int b = s; b < G; b += 8 * S) {
+        double v[CC][8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+#pragma unroll
+            for (int c = 0; c < CC; ++c)
+                v[c][r] = b + r * S < G ? __ldcg(ws + (int64_t)(b + r * S) * stride + o * CC + c) : 0.0;
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+            if (b + r * S < G)
+#pragma unroll
+                for (int c = 0; c < CC; ++c) acc[c][r] += v[c][r];
+    }
+#pragma unroll
+    for (int c = 0; c < CC; ++c)
+        out[c] = ((acc[c][0] + acc[c][1]) + (acc[c][2] + acc[c][3])) +
+                 ((acc[c][4] + acc[c][5]) + (acc[c][6] + acc[c][7]));
+}
+
 // Warp-level sum of V values per lane (V a power of two, 1 <= V <= 32) by
 // recursive halving: at the step with lane offset o = 16, 8, ..., a lane
 // keeps half of its remaining values (the upper half if its bit o is set)

@@ -260,9 +260,16 @@ namespace {
 // tree), the S slice sums are combined by a fixed shuffle tree, and the
 // first lane stores alpha * sum + beta * C.  With S chosen so that each
 // lane takes a few dozen partials, the pass is a handful of L2 round trips
-// however many CTAs wrote partials.
+// however many CTAs wrote partials.  Small CTAs spread those over more SMs:
+// complex 8 x 8, 10^5 rows 55.3 us a call with CTAs of 256 threads, 53.2 with
+// 64.  Behind a short product the launch may start early whatever its size,
+// its few CTAs only wait (complex 8 x 8, 3000 rows: 11 us a call, 14 without);
+// behind a long one that lets the product after it start too soon, on SMs
+// that free up unevenly (the Gram-Schmidt step of complex 60 x 4, 10^6 rows,
+// 3.29 ms instead of 3.16).
+constexpr int kFinalBlock = 64;
 template <int CC>
-__global__ void __launch_bounds__(256) k_tsmttsm_final(const TsmttsmArgs a, int G, int S) {
+__global__ void __launch_bounds__(kFinalBlock) k_tsmttsm_final(const TsmttsmArgs a, int G, int S) {
     pdl_trigger();
     pdl_wait();  // the partials of the launch before
     const int MN = a.M * a.N;
@@ -270,7 +277,7 @@ __global__ void __launch_bounds__(256) k_tsmttsm_final(const TsmttsmArgs a, int 
     const int o = gt / S, s = gt - o * S;  // S divides 32: an entry's lanes share a warp
     double v[CC];
     if (o < MN) {
-        sum_partials<CC>(a.ws, MN * CC, o, G, s, S, v);
+        sum_partials_batched<CC>(a.ws, MN * CC, o, G, s, S, v);
     } else {
 #pragma unroll
         for (int c = 0; c < CC; ++c) v[c] = 0.0;
@@ -284,13 +291,14 @@ __global__ void __launch_bounds__(256) k_tsmttsm_final(const TsmttsmArgs a, int 
 }  // namespace
 
 cudaError_t launch_tsmttsm_final(const TsmttsmArgs& a, int grid, int cplx, cudaStream_t s) {
+    const bool early = short_product(a.M, a.N, a.K, cplx) && pdl_enabled();
     const int MN = a.M * a.N;
     int S = 1;
     while (S < 32 && grid >= 16 * S) S *= 2;  // at least 8 partials per lane
     const int threads = MN * S;
-    const int blocks = (threads + 255) / 256;
-    if (cplx) return launch_pdl(k_tsmttsm_final<2>, blocks, 256, 0, s, a, grid, S);
-    return launch_pdl(k_tsmttsm_final<1>, blocks, 256, 0, s, a, grid, S);
+    const int blocks = (threads + kFinalBlock - 1) / kFinalBlock;
+    if (cplx) return launch_early(early, k_tsmttsm_final<2>, blocks, kFinalBlock, 0, s, a, grid, S);
+    return launch_early(early, k_tsmttsm_final<1>, blocks, kFinalBlock, 0, s, a, grid, S);
 }
 
 cudaError_t launch_scale_small(double* C, int rows, int cols, int64_t ld, int cplx, double br, double bi,

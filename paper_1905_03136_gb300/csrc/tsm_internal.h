@@ -61,9 +61,13 @@ bool pdl_enabled();
 // taking several, and a grid sized for k CTAs per SM would run unevenly.
 bool pdl_allowed(const void* kernel, int grid, int block, size_t smem);
 
+// Resident CTAs per SM of a kernel at a CTA size and dynamic shared memory
+// on the current device (the occupancy query's answer, kept; 0 if it fails).
+int resident_ctas(const void* kernel, int block, size_t smem);
+
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s,
-                       Args... args) {
+cudaError_t launch_early(bool early, void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s,
+                         Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)block);
@@ -73,20 +77,31 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t sme
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = pdl_allowed((const void*)kernel, grid, block, smem) ? 1 : 0;
+    cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s,
+                       Args... args) {
+    return launch_early(pdl_allowed((const void*)kernel, grid, block, smem), kernel, grid, block, smem, s, args...);
 }
 
 typedef cudaError_t (*TsmttsmLaunch)(const TsmttsmArgs&, int grid, cudaStream_t);
 typedef cudaError_t (*TsmmLaunch)(const TsmmArgs&, int grid, cudaStream_t);
 // Resident CTAs per SM for this variant and shape (0 if it cannot run).
 typedef int (*OccupancyFn)(int M, int N);
+// Default grid of a variant that does not want full residency at every K.
+typedef int (*GridFn)(int M, int N, int64_t K);
 
 struct Variant {
     tsm_variant_info info;
     TsmttsmLaunch tsmttsm;  // exactly one of the two launchers is set
     TsmmLaunch tsmm;
     OccupancyFn occupancy;
+    GridFn grid;                    // may be null: occupancy x SMs
+    bool (*supports)(int M, int N); // may be null: the info's fields decide
+    bool final_pass;                // partials always summed by the final kernel
 };
 
 // Variant tables, filled once in a fixed order (indices are stable within a
@@ -95,6 +110,7 @@ void register_fp64_variants(std::vector<Variant>& tsmttsm, std::vector<Variant>&
 void register_generated_variants(std::vector<Variant>& tsmttsm, std::vector<Variant>& tsmm);
 void register_rt_variants(std::vector<Variant>& tsmttsm, std::vector<Variant>& tsmm);
 void register_narrow_variants(std::vector<Variant>& tsmttsm, std::vector<Variant>& tsmm);
+void register_row_variants(std::vector<Variant>& tsmttsm);
 
 // Second pass of the TSMTTSM reduction when the partials are many
 // (grid * M * N * c > kFinalThreshold doubles): one thread per entry of C
@@ -102,7 +118,15 @@ void register_narrow_variants(std::vector<Variant>& tsmttsm, std::vector<Variant
 // over ceil(M*N / 128) CTAs, this replaces the last CTA's single-SM sum,
 // whose FP64 adds alone would take grid * M*N*c / 2 cycles on this part.
 constexpr int kFinalThreshold = 32768;
+// Products whose time is mostly launch, load latency and reduction.
+inline bool short_product(int M, int N, int64_t K, int cplx) {
+    return (double)M * N * (cplx ? 4 : 1) * (double)K <= 1e8;
+}
 cudaError_t launch_tsmttsm_final(const TsmttsmArgs& a, int grid, int cplx, cudaStream_t s);
+
+// Index-independent part of the row kernel's rule (kernels_row.cu): the FP64
+// slots its tile takes per useful FMA, 0 if it cannot run the shape.
+double row_slots(int M, int N, int cplx);
 
 // Per-launch choice of the runtime-threads-per-row TSMM variants (kernels_rt.cu).
 void rt_tsmm_tpr(int N, int nptmax, int* tpr, int* npt);

@@ -74,7 +74,7 @@ int k_bucket(int64_t K) {
     return b;
 }
 
-tsm_status tune_lookup(int kind, int dtype, int M, int N, int64_t K, int* variant, int* grid) {
+tsm_status tune_lookup(int kind, int dtype, int M, int N, int64_t K, int* variant, int* grid, int* distance) {
     std::lock_guard<std::mutex> lock(g_mu);
     if (!g_env_loaded) {
         g_env_loaded = true;
@@ -103,6 +103,7 @@ tsm_status tune_lookup(int kind, int dtype, int M, int N, int64_t K, int* varian
     if (v < 0) return TSM_ERR_NOT_SUPPORTED;
     *variant = v;
     *grid = best->grid;
+    if (distance) *distance = best_d;
     return TSM_OK;
 }
 

@@ -7,7 +7,8 @@
 namespace tsm {
 
 // Looks up (kind, dtype, M, N, K bucket); TSM_OK with *variant >= 0 on a hit.
-tsm_status tune_lookup(int kind, int dtype, int M, int N, int64_t K, int* variant, int* grid);
+tsm_status tune_lookup(int kind, int dtype, int M, int N, int64_t K, int* variant, int* grid,
+                       int* distance = nullptr);
 
 const Variant* variant_at(tsm_kind kind, int idx);
 bool supports(tsm_kind kind, int idx, int dtype, int M, int N);
