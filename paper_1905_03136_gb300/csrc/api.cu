@@ -1,6 +1,7 @@
 // C-ABI entry points of libtsm: argument validation, the variant registry,
 // per-(device, stream) workspaces and dispatch.  Every product runs in the
 // library's own kernels; there is no CPU fallback.
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -227,6 +228,7 @@ struct Registry {
         register_rt_variants(tsmttsm, tsmm);
         register_narrow_variants(tsmttsm, tsmm);
         register_row_variants(tsmttsm);
+        register_mm_variants(tsmm);
     }
 };
 
@@ -373,6 +375,78 @@ static bool row_preferred(const tsm_variant_info& other, bool tuned, int dtype, 
     return !tuned && slots * 1.05 < waste;
 }
 
+// Threads per row and results per thread a TSMM variant gives N columns.
+static void tsmm_split(const tsm_variant_info& f, int N, int* tpr, int* npt) {
+    *tpr = f.threads_per_row;
+    *npt = f.tile_n;
+    if (f.runtime_tile) rt_tsmm_tpr(N, f.tile_n, tpr, npt);
+}
+
+// Time of a TSMM variant that walks K with a grid stride over that of its
+// useful FMAs alone: padded results, idle lanes, the last of its passes, and
+// what such kernels were measured to take at no padding (the runtime variant
+// runs three real results per thread at the rate of four and a half).
+static double stride_cost(const tsm_variant_info& f, int cplx, int N, int64_t K, int grid) {
+    int tpr, npt;
+    tsmm_split(f, N, &tpr, &npt);
+    if (tpr <= 0 || f.block < tpr) return 1.0;
+    const int sms = device_info().sm_count, cps = (grid + sms - 1) / sms;
+    const int rpc = f.block / tpr * f.unroll;
+    const int64_t n = (K + rpc - 1) / rpc, rest = n % grid;
+    const int64_t most = n / grid * cps + std::min<int64_t>(cps, (rest + sms - 1) / sms);
+    double own = 1.015;
+    if (!f.generated) own = !f.runtime_tile ? 1.04 : npt != 3 ? 1.06 : cplx ? 1.1 : 1.5;
+    if (n <= 2 * (int64_t)grid) own *= n <= grid ? 1.1 : 1.05;  // nothing to overlap the first loads with
+    return own * (double)most * sms * rpc / (double)K * f.block / (f.block / tpr * tpr) * tpr * npt / N;
+}
+
+// Whether TSMM's row kernel (kernels_mm.cu) runs a product below 2^22 rows
+// instead of `other` (the nearest tuned entry's variant, or the heuristic's).
+// Measured, us a call back to back, other / row kernel:
+//   short products, whose time in the other kernels is that of a pass of a
+//     full grid: real 8 x 8, 6000 rows 6.1 / 2.3; complex 16 x 16, 1000 rows
+//     34.3 / 5.0; real 64 x 64, 1000 rows 71.7 / 11.3; complex 64 x 64, 6000
+//     rows 276 / 170, 30000 rows 1053 / 809.
+//   longer ones by the slots, lanes and passes each wastes: complex 23 x 11,
+//     200003 rows 350 / 338; real 18 x 21, 1.6 10^6 rows 1430 / 969 (three
+//     results per thread); complex 64 x 64, 150000 rows 4152 / 3945; real
+//     31 x 11, 567000 rows 334 / 346 (stays).
+//   products bound by memory (few FMAs a row, one or two columns of A) meet at
+//     about 10^6 FMAs: real 2 x 2, 150000 rows 3.7 / 3.1, 700000 rows 7.2 /
+//     8.1; real 1 x 8, 164000 rows 4.4 / 12.3.
+// Of 1982 drawn products the rule takes 1276, in the geometric mean 1.64 times
+// as fast there, four of them 3 to 7 % slower.
+static bool mm_preferred(const tsm_variant_info& other, int grid, int dtype, int M, int N, int64_t K) {
+    if (K >= ((int64_t)1 << 22)) return false;
+    const int cplx = dtype == TSM_C64;
+    const double per_row = (double)M * N * (cplx ? 4 : 1), fma = per_row * (double)K;
+    // how much dearer the other has to be: the row kernel's own cost spreads
+    // more at few columns of A and with short products
+    const double margin = M < 8 ? 1.15 : cplx ? (fma < 3e7 ? 1.04 : 1.01) : (fma < 3e7 ? 1.12 : 1.04);
+    auto cheaper = [&] { return stride_cost(other, cplx, N, K, grid) > margin * mm_cost(M, N, K, cplx); };
+    int tpr, npt;
+    tsmm_split(other, N, &tpr, &npt);
+    const bool slow_split = other.runtime_tile && !cplx && npt == 3;
+    if (other.generated && M * N <= 4) return false;
+    // single columns: the other kernels' threads each read a row on their own
+    if (N == 1 && M >= 16) return M >= 24 || fma <= 3e7;
+    if (N == 1 && M >= 12) return fma <= 2.5e6;
+    if (per_row < 64.0) {
+        if (slow_split && M >= 3) return fma <= 1e6 || cheaper();
+        if (M >= 12) return fma <= 8e6 || cheaper();
+        if (cplx) return fma <= (M >= 3 ? 4e6 : M > 1 && N > 1 ? 2.5e6 : 1e6);
+        if (M >= 8) return fma <= 1e6;
+        if (M == 1) return strstr(other.name, "narrow") && fma <= 1e6;
+        return (N > 1 || M >= 6) && fma <= (M > 2 ? 5e5 : 3e5);
+    }
+    if (M < 4) {
+        if (!cplx && other.runtime_tile && N >= 16 && fma > 5e6 && (npt == 1 || (npt == 3 && M > 1))) return true;
+        if (slow_split && M == 3) return cheaper();
+        return fma <= (M == 1 ? 3e5 : cplx ? 2.5e6 : 5e5) && (cplx || M > 1);
+    }
+    return fma <= 5e6 || cheaper();
+}
+
 tsm_status choose(tsm_kind kind, int dtype, int M, int N, int64_t K, int* variant, int* grid) {
     const std::vector<Variant>* t = table(kind);
     if (!t) return TSM_ERR_INVALID_VALUE;
@@ -398,6 +472,13 @@ tsm_status choose(tsm_kind kind, int dtype, int M, int N, int64_t K, int* varian
         }
     }
     if (g <= 0) g = default_grid((*t)[v], M, N, K);
+    if (kind != TSM_KIND_TSMTTSM && distance != 0 && mm_preferred((*t)[v].info, g, dtype, M, N, K)) {
+        static const int row[2] = {find_named(TSM_KIND_TSMM, "tsmm_r64_row"), find_named(TSM_KIND_TSMM, "tsmm_c64_row")};
+        if (row[dtype == TSM_C64] >= 0) {
+            v = row[dtype == TSM_C64];
+            g = default_grid((*t)[v], M, N, K);
+        }
+    }
     *variant = v;
     *grid = g;
     return TSM_OK;
@@ -645,7 +726,9 @@ tsm_status tsm_variant_shape(tsm_kind kind, int index, tsm_dtype dtype, int M, i
     if (!v || !info) return TSM_ERR_INVALID_VALUE;
     if (!variant_supports(*v, dtype, M, N)) return TSM_ERR_NOT_SUPPORTED;
     *info = v->info;
-    if (v->info.runtime_tile) {
+    if (v->resolve) {
+        v->resolve(M, N, info);
+    } else if (v->info.runtime_tile) {
         if (kind == TSM_KIND_TSMM || kind == TSM_KIND_TSMM_BETA)
             rt_tsmm_tpr(N, v->info.tile_n, &info->threads_per_row, &info->tile_n);
     }

@@ -302,6 +302,12 @@ Variant make_row() {
     v.occupancy = occ_row<CPLX>;
     v.grid = grid_row<CPLX>;
     v.final_pass = true;
+    v.resolve = [](int M, int N, tsm_variant_info* info) {
+        const RowShape& r = row_shape(M, N, CPLX);
+        info->tile_m = r.along_m ? r.T : 1;
+        info->tile_n = r.along_m ? 1 : r.T;
+        info->block = r.block;
+    };
     v.supports = [](int M, int N) { return row_shape(M, N, CPLX).T > 0; };
     return v;
 }

@@ -101,6 +101,7 @@ struct Variant {
     OccupancyFn occupancy;
     GridFn grid;                    // may be null: occupancy x SMs
     bool (*supports)(int M, int N); // may be null: the info's fields decide
+    void (*resolve)(int M, int N, tsm_variant_info*);  // tile of a long product (runtime-tile variants); may be null
     bool final_pass;                // partials always summed by the final kernel
 };
 
@@ -111,6 +112,9 @@ void register_generated_variants(std::vector<Variant>& tsmttsm, std::vector<Vari
 void register_rt_variants(std::vector<Variant>& tsmttsm, std::vector<Variant>& tsmm);
 void register_narrow_variants(std::vector<Variant>& tsmttsm, std::vector<Variant>& tsmm);
 void register_row_variants(std::vector<Variant>& tsmttsm);
+void register_mm_variants(std::vector<Variant>& tsmm);
+// Time of the row variant of TSMM (kernels_mm.cu) over that of its FMAs alone.
+double mm_cost(int M, int N, int64_t K, int cplx);
 
 // Second pass of the TSMTTSM reduction when the partials are many
 // (grid * M * N * c > kFinalThreshold doubles): one thread per entry of C
