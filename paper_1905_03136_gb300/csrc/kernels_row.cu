@@ -247,18 +247,18 @@ template <bool CPLX>
 cudaError_t launch_row(const TsmttsmArgs& a, int grid, cudaStream_t s) {
     const RowShape& r = row_shape(a.M, a.N, CPLX);
     const Kernel k = kernel_for<CPLX>(r.T, a.conj != 0);
-    // the shortest start early at any grid: one CTA per SM is soon placed
-    if (row_work(a.M, a.N, a.K, CPLX) < 1e7)
-        return launch_early(pdl_enabled(), k, grid, r.block, 0, s, a, r.along_m, r.P, r.L);
-    const int sms = device_info().sm_count, cps = grid / sms;
+    const int sms = device_info().sm_count, cps = (grid + sms - 1) / sms;
     size_t smem = 0;
-    if (grid % sms == 0 && cps >= 1 && cps < resident_ctas((const void*)k, r.block, 0)) {
+    if (cps < resident_ctas((const void*)k, r.block, 0)) {
         smem = limit_smem(cps);
         if (smem > 48 * 1024) {
             const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
     }
+    // the shortest start early at any grid: one CTA per SM is soon placed
+    if (row_work(a.M, a.N, a.K, CPLX) < 1e7)
+        return launch_early(pdl_enabled(), k, grid, r.block, smem, s, a, r.along_m, r.P, r.L);
     return launch_pdl(k, grid, r.block, smem, s, a, r.along_m, r.P, r.L);
 }
 
@@ -268,18 +268,23 @@ int occ_row(int M, int N) {
     return resident_ctas((const void*)kernel_for<CPLX>(r.T, false), r.block, 0);
 }
 
-// CTAs per SM by the work: one below 10^7 FMAs, or where two would leave a CTA
-// fewer than 64 rows for its partial; two below 10^8; else what fits.
+// CTAs per SM by the work: one below 6 10^6 FMAs (3 10^6 if a CTA has no more
+// than six warps to hide its loads with), or where two would leave a CTA of
+// more fewer than 64 rows for its partial; two below 10^8; else what fits.
 // Measured (us, one / two / what fits): real 6 x 6 at 50000 rows 9.1 / 10.6 /
 // 16.7, complex 50 x 50 at 5000 rows 99.6 / 108 / 99.6, real 22 x 22 at 52291
-// rows 80.6 / 52.7 / 60.6, complex 17 x 33 at 200000 rows 1211 / 849 / 788.
+// rows 80.6 / 52.7 / 60.6, complex 17 x 33 at 200000 rows 1211 / 849 / 788;
+// one / two: real 43 x 17 (192 threads) at 9575 rows 26.6 / 19.9, real 16 x 16
+// at 27343 rows 21.8 / 19.5, real 8 x 8 at 109375 rows 21.7 / 19.0, complex
+// 16 x 16 at 3906 rows 11.4 / 13.6, complex 32 x 32 at 4882 rows 42.1 / 43.8.
 template <bool CPLX>
 int grid_row(int M, int N, int64_t K) {
     const int sms = device_info().sm_count;
     const int occ = std::max(occ_row<CPLX>(M, N), 1);
     const double fma = row_work(M, N, K, CPLX);
     int cps = occ;
-    if (fma < 1e7 || K < 128 * (int64_t)sms)
+    const bool few_warps = row_shape(M, N, CPLX).block <= 192;
+    if (fma < (few_warps ? 3e6 : 6e6) || (!few_warps && K < 128 * (int64_t)sms))
         cps = 1;
     else if (fma < 1e8)
         cps = 2;
