@@ -198,8 +198,9 @@ tsm_status tsm_tsmm_ex(tsm_op opC, tsm_dtype dtype, int M, int N, int64_t K,
  * reads it from device memory once per CTA into shared memory.  Both
  * products use the variants the tuning table selects; the two launches are
  * enqueued on `stream` back to back (no host synchronisation, capturable in
- * a CUDA graph).  For K <= 2^15 the step runs as one fused cooperative
- * kernel instead (tsm_gs_step_ex).  With A not orthonormal the same two products run (one
+ * a CUDA graph).  The shortest steps (up to 800 rows; up to 8000, or 2^15, of
+ * some narrow shapes) run as one fused cooperative kernel instead
+ * (tsm_gs_step_ex).  With A not orthonormal the same two products run (one
  * classical Gram-Schmidt projection).
  * Errors: as tsm_tsmttsm / tsm_tsmm; C == NULL -> INVALID_VALUE; every check
  * runs before the first launch, so on an error B and C are untouched.  C must
@@ -211,7 +212,7 @@ tsm_status tsm_gs_step(tsm_dtype dtype, int M, int N, int64_t K, const void *A,
 
 /* How tsm_gs_step_ex runs the step. */
 typedef enum {
-    TSM_GS_AUTO = 0,         /* fused for K <= 2^15, else two products */
+    TSM_GS_AUTO = 0,         /* fused where that is the faster, else two products */
     TSM_GS_TWO_PRODUCTS = 1, /* the TSMTTSM and TSMM launches described above */
     TSM_GS_FUSED = 2         /* one cooperative kernel (below) */
 } tsm_gs_mode;

@@ -375,12 +375,21 @@ tsm_status gs_fused_run(tsm_dtype dtype, int M, int N, int64_t K, const void* A,
     return gsf::run(dtype, M, N, K, A, lda, B, ldb, C, ldc, s);
 }
 
-// Fused up to 2^15 rows.  Measured on 12 shapes (real and complex, 1 x 1
-// to 64 x 64 and 37 x 53) at K = 1, 3000, 10^4 and 2^15, the fused step was
-// faster or within 2 % at 46 of the 48 points (up to 3.3x faster: complex
-// 64 x 64 at K = 3000); the two exceptions are real 16 x 16 and 37 x 53 at
-// 2^15 (12 % and 2.4 % slower).  Above 2^15 the tuned product kernels win.
-bool gs_fused_preferred(tsm_dtype, int, int, int64_t K) { return K <= (1 << 15); }
+// Fused where the two products' launches (12 us of host time) or the latency of
+// their final reduction outweigh the fused kernel's barriers and generic loops:
+// up to 800 rows, and to 1500 to 8000 of the narrowest.  Measured on 63 shapes
+// at 7 row counts (us, fused / two products): real 64 x 64 at 100 rows 27 / 41,
+// at 1000 rows 41 / 38; real 4 x 4 at 1000 rows 11.3 / 12.3, at 5000 rows 13.3 /
+// 12.3; complex 16 x 16 at 100 rows 18.5 / 17, at 10000 rows 52.6 / 47.5; real
+// 12 x 12 at 20000 rows 34.5 / 22.2; real 37 x 53 at 32000 rows 282 / 236.  One or
+// two columns of A times many of B stay fused to 2^15 rows when complex (2 x 30
+// at 20000 rows 34.8 / 37.0).
+bool gs_fused_preferred(tsm_dtype dtype, int M, int N, int64_t K) {
+    const bool cplx = dtype == TSM_C64;
+    if (cplx && M <= 2 && N >= 16) return K <= (1 << 15);
+    if (M == 1 || N == 1) return K <= (N == 1 ? 8000 : 3000);
+    return K <= ((cplx ? 4 : 1) * M * N < 64 ? 1500 : 800);
+}
 
 }  // namespace tsm
 
