@@ -342,8 +342,7 @@ static double tile_slots(const tsm_variant_info& f, int M, int N) {
     return (double)((P * L + 31) / 32 * 32) * f.tile_m * f.tile_n / ((double)L * M * N);
 }
 
-// Whether the row kernel (kernels_row.cu) runs a product below 2^21 rows
-// instead of `other` (the nearest tuned entry's variant, or the heuristic's).
+// Whether the row kernel (kernels_row.cu) runs a product instead of `other` (the nearest tuned entry's variant, or the heuristic's).
 // Measured, us a call, other / row kernel:
 //   up to 10^8 FMAs, whose time is mostly the other kernels' reduction tails:
 //     real 8 x 8, 16000 rows 16.4 / 10.2; real 6 x 6, 50000 rows 48 / 9.1; complex
@@ -361,13 +360,28 @@ static double tile_slots(const tsm_variant_info& f, int M, int N) {
 //   longer products without a tuned entry, by the slots their tiles waste:
 //     real 37 x 53, 300007 rows 1119 / 999 (1.14 against 1.03); complex 17 x 33,
 //     200000 rows 880 / 788; real 9 x 41, 10^6 rows 671 / 690 (1.04, 1.03: stays).
-static bool row_preferred(const tsm_variant_info& other, bool tuned, int dtype, int M, int N, int64_t K) {
+//   from 2^21 rows on only where a loaded table has no entry of the shape (an
+//     empty table's plain heuristic is what the cost model is judged against),
+//     by the slots and by what the other's tile takes at no waste: complex
+//     45 x 32, 1.6 10^7 rows 1.20 times as fast, real 58 x 13 1.20, real 7 x 5
+//     1.22, complex 53 x 11 1.14; real 41 x 9 0.95, complex 50 x 13 0.95.
+static bool row_preferred(const tsm_variant_info& other, int distance, int dtype, int M, int N, int64_t K) {
     const double slots = row_slots(M, N, dtype == TSM_C64);
-    if (slots <= 0.0 || K >= ((int64_t)1 << 21)) return false;
+    if (slots <= 0.0) return false;
+    const bool tuned = distance > 0;
     const double per_row = (double)M * N * (dtype == TSM_C64 ? 4 : 1), fma = per_row * (double)K;
     const bool narrow = strstr(other.name, "narrow") != nullptr;
     const double waste = narrow ? 1.0 : tile_slots(other, M, N);
     const bool small_tile = narrow || (!other.generated && other.tile_m * other.tile_n <= 4);
+    if (K >= ((int64_t)1 << 21)) {
+        if (distance != -1 || other.generated || narrow || M == 1 || N == 1 || per_row < 32.0) return false;
+        // time over slots of the other's tile (its loads per FMA) and of the strip
+        const int area = other.tile_m * other.tile_n;
+        const bool cplx = dtype == TSM_C64;
+        const double theirs = cplx ? (area == 1 ? 1.08 : 1.05) : area == 1 ? 1.25 : area < 16 ? 1.09 : 1.05;
+        const double own = cplx ? 1.05 : row_block(M, N, 0) <= 192 ? 1.2 : 1.09;
+        return waste * theirs > 1.04 * slots * own;
+    }
     if (narrow && fma < 5e5) return false;
     if (per_row < 64.0 && small_tile && waste < 1.3)
         return fma <= 5e6 && 8.0 * (dtype == TSM_C64 ? 2 : 1) * (M + N) * (double)K <= 1.7e7;
@@ -400,8 +414,10 @@ static double stride_cost(const tsm_variant_info& f, int cplx, int N, int64_t K,
     return own * (double)most * sms * rpc / (double)K * f.block / (f.block / tpr * tpr) * tpr * npt / N;
 }
 
-// Whether TSMM's row kernel (kernels_mm.cu) runs a product below 2^22 rows
-// instead of `other` (the nearest tuned entry's variant, or the heuristic's).
+// Whether TSMM's row kernel (kernels_mm.cu) runs a product instead of `other`
+// (the nearest tuned entry's variant, or the heuristic's).  With an empty
+// tuning table the plain heuristic stands from 2^22 rows on: the cost model is
+// judged against it there.
 // Measured, us a call back to back, other / row kernel:
 //   short products, whose time in the other kernels is that of a pass of a
 //     full grid: real 8 x 8, 6000 rows 6.1 / 2.3; complex 16 x 16, 1000 rows
@@ -414,23 +430,31 @@ static double stride_cost(const tsm_variant_info& f, int cplx, int N, int64_t K,
 //   products bound by memory (few FMAs a row, one or two columns of A) meet at
 //     about 10^6 FMAs: real 2 x 2, 150000 rows 3.7 / 3.1, 700000 rows 7.2 /
 //     8.1; real 1 x 8, 164000 rows 4.4 / 12.3.
-// Of 1982 drawn products the rule takes 1276, in the geometric mean 1.64 times
+//   real 1 x 35, 1.6 10^7 rows (one result per thread): 1.59 times as fast; real
+//     6 x 47, 8 10^6 rows 1.13; real 36 x 3, 10^7 rows 2735 / 1890.
+//   Over 119 products from 2^22 rows on that the two rules take: 1.144 times as
+//     fast in the geometric mean, the worst 0.95.
+// Of 1982 drawn products below 2^22 rows the rule takes 1276, in the geometric mean 1.64 times
 // as fast there, four of them 3 to 7 % slower.
-static bool mm_preferred(const tsm_variant_info& other, int grid, int dtype, int M, int N, int64_t K) {
-    if (K >= ((int64_t)1 << 22)) return false;
+static bool mm_preferred(const tsm_variant_info& other, int grid, int distance, int dtype, int M, int N, int64_t K) {
+    if (K >= ((int64_t)1 << 22) && distance == -2) return false;
     const int cplx = dtype == TSM_C64;
     const double per_row = (double)M * N * (cplx ? 4 : 1), fma = per_row * (double)K;
-    // how much dearer the other has to be: the row kernel's own cost spreads
-    // more at few columns of A and with short products
-    const double margin = M < 8 ? 1.15 : cplx ? (fma < 3e7 ? 1.04 : 1.01) : (fma < 3e7 ? 1.12 : 1.04);
-    auto cheaper = [&] { return stride_cost(other, cplx, N, K, grid) > margin * mm_cost(M, N, K, cplx); };
     int tpr, npt;
     tsmm_split(other, N, &tpr, &npt);
+    // how much dearer the other has to be: the row kernel's own cost spreads
+    // more at few columns of A and with short products
+    const bool plain_rt = other.runtime_tile && npt < 3 && fma >= 3e7;
+    const double margin = M < 8 ? (plain_rt ? 1.04 : 1.15) : cplx ? (fma < 3e7 ? 1.04 : 1.015) : (fma < 3e7 ? 1.12 : 1.04);
+    auto cheaper = [&] { return stride_cost(other, cplx, N, K, grid) > margin * mm_cost(M, N, K, cplx); };
     const bool slow_split = other.runtime_tile && !cplx && npt == 3;
     if (other.generated && M * N <= 4) return false;
     // single columns: the other kernels' threads each read a row on their own
-    if (N == 1 && M >= 16) return M >= 24 || fma <= 3e7;
+    if (N == 1 && M >= 16) return M >= (fma <= 1e8 ? 24 : 32) || fma <= 3e7;
     if (N == 1 && M >= 12) return fma <= 2.5e6;
+    // one to three columns of A, and results that the runtime variant gives a
+    // thread each: its loads of A bound it
+    if (M < 4 && !cplx && other.runtime_tile && N >= 16 && fma > 5e6 && (npt == 1 || (npt == 3 && M > 1))) return true;
     if (per_row < 64.0) {
         if (slow_split && M >= 3) return fma <= 1e6 || cheaper();
         if (M >= 12) return fma <= 8e6 || cheaper();
@@ -440,7 +464,6 @@ static bool mm_preferred(const tsm_variant_info& other, int grid, int dtype, int
         return (N > 1 || M >= 6) && fma <= (M > 2 ? 5e5 : 3e5);
     }
     if (M < 4) {
-        if (!cplx && other.runtime_tile && N >= 16 && fma > 5e6 && (npt == 1 || (npt == 3 && M > 1))) return true;
         if (slow_split && M == 3) return cheaper();
         return fma <= (M == 1 ? 3e5 : cplx ? 2.5e6 : 5e5) && (cplx || M > 1);
     }
@@ -459,11 +482,11 @@ tsm_status choose(tsm_kind kind, int dtype, int M, int N, int64_t K, int* varian
     if (!looked_up(kind) && !(kind == TSM_KIND_TSMM_BETA && looked_up(TSM_KIND_TSMM))) {
         v = heuristic_variant(kind == TSM_KIND_TSMM_BETA ? TSM_KIND_TSMM : kind, dtype, M, N);
         g = 0;
-        distance = -1;
+        if (distance >= 0) distance = -1;  // (-2: the table is empty)
     }
     if (v < 0) return TSM_ERR_NOT_SUPPORTED;
     // an entry tuned for this very bucket of K stands
-    if (kind == TSM_KIND_TSMTTSM && distance != 0 && row_preferred((*t)[v].info, distance > 0, dtype, M, N, K)) {
+    if (kind == TSM_KIND_TSMTTSM && distance != 0 && row_preferred((*t)[v].info, distance, dtype, M, N, K)) {
         static const int row[2] = {find_named(TSM_KIND_TSMTTSM, "tsmttsm_r64_row"),
                                    find_named(TSM_KIND_TSMTTSM, "tsmttsm_c64_row")};
         if (row[dtype == TSM_C64] >= 0) {
@@ -472,7 +495,7 @@ tsm_status choose(tsm_kind kind, int dtype, int M, int N, int64_t K, int* varian
         }
     }
     if (g <= 0) g = default_grid((*t)[v], M, N, K);
-    if (kind != TSM_KIND_TSMTTSM && distance != 0 && mm_preferred((*t)[v].info, g, dtype, M, N, K)) {
+    if (kind != TSM_KIND_TSMTTSM && distance != 0 && mm_preferred((*t)[v].info, g, distance, dtype, M, N, K)) {
         static const int row[2] = {find_named(TSM_KIND_TSMM, "tsmm_r64_row"), find_named(TSM_KIND_TSMM, "tsmm_c64_row")};
         if (row[dtype == TSM_C64] >= 0) {
             v = row[dtype == TSM_C64];

@@ -320,6 +320,7 @@ Variant make_row() {
 }  // namespace
 
 double row_slots(int M, int N, int cplx) { return row_shape(M, N, cplx).slots; }
+int row_block(int M, int N, int cplx) { return row_shape(M, N, cplx).block; }
 
 void register_row_variants(std::vector<Variant>& tsmttsm) {
     tsmttsm.push_back(make_row<false>());

@@ -95,7 +95,10 @@ tsm_status tune_lookup(int kind, int dtype, int M, int N, int64_t K, int* varian
             best = &it->second;
         }
     }
-    if (!best) return TSM_ERR_NOT_SUPPORTED;
+    if (!best) {
+        if (distance) *distance = g_table.empty() ? -2 : -1;
+        return TSM_ERR_NOT_SUPPORTED;
+    }
     // the name is resolved once per entry: a scan of a few hundred variant
     // names per call would cost microseconds of host time
     if (best->index == -2) best->index = find_variant(kind, best->name);

@@ -63,12 +63,18 @@ def test_row_kernel(tsm, shape, cplx):
 
 def test_rule_for_short_products(tsm):
     """Short products take the row kernels (the very shortest of the narrow
-    widths do not), products from 2^21 rows on never do, and an entry tuned for the very bucket of K stands."""
+    widths do not), products from 2^21 rows on only without an entry for their
+    shape in a table that has others, and an entry tuned for the very bucket
+    of K stands."""
+    from paper_1905_03136_gb300 import costmodel as cm
     rows = (_row(tsm, False), _row(tsm, True))
-    for cplx, M, N, K in [(0, 4, 4, 60000), (1, 8, 8, 100000), (0, 25, 25, 60000), (0, 37, 53, 300007)]:
+    for cplx, M, N, K in [(0, 4, 4, 60000), (1, 8, 8, 100000), (0, 25, 25, 60000), (0, 37, 53, 300007),
+                          (0, 58, 13, 1 << 23), (1, 45, 32, 1 << 22)]:
         assert tsm.choose(tsm.KIND_TSMTTSM, cplx, M, N, K)[0] == rows[cplx], (cplx, M, N, K)
-    for cplx, M, N, K in [(0, 4, 4, 1 << 21), (0, 4, 4, 10000), (1, 64, 64, 5000), (0, 37, 53, 1 << 22), (0, 4, 4, 900000)]:
+    for cplx, M, N, K in [(0, 4, 4, 1 << 21), (0, 4, 4, 10000), (1, 64, 64, 5000), (0, 9, 1, 1 << 23), (0, 4, 4, 900000)]:
         assert tsm.choose(tsm.KIND_TSMTTSM, cplx, M, N, K)[0] != rows[cplx], (cplx, M, N, K)
+    for cplx, M, N in [(0, 58, 13), (1, 45, 32)]:
+        assert not cm.heuristic_pick(tsm.KIND_TSMTTSM, cplx, M, N, 1 << 22)[0].endswith("_row")
     lib = tsm.load()
     other = [v["index"] for v in tsm.variants(tsm.KIND_TSMTTSM) if v["name"] == "tsmttsm_r64_direct_t1x1_u4"][0]
     assert lib.tsm_set_tuning(tsm.KIND_TSMTTSM, 0, 11, 6, 5000, other, 152) == 0

@@ -63,14 +63,17 @@ def test_row_kernel(tsm, shape, cplx):
 
 def test_rule(tsm):
     """Short products, and longer ones whose other kernel pads or leaves the
-    chip idle, take the row kernel; from 2^22 rows on none does; products bound
-    by memory do not; an entry tuned for the very bucket of K stands."""
+    chip idle, take the row kernel; from 2^22 rows on none does without a
+    tuning table; products bound by memory do not; an entry tuned for the very
+    bucket of K stands."""
+    from paper_1905_03136_gb300 import costmodel as cm
     rows = (_row(tsm, False), _row(tsm, True))
-    for cplx, M, N, K in [(1, 64, 64, 1000), (0, 8, 8, 6000), (1, 23, 11, 200003), (0, 18, 21, 1500000)]:
+    for cplx, M, N, K in [(1, 64, 64, 1000), (0, 8, 8, 6000), (1, 23, 11, 200003), (0, 18, 21, 1500000), (0, 36, 3, 10000000)]:
         for kind in (tsm.KIND_TSMM, tsm.KIND_TSMM_BETA):
             assert tsm.choose(kind, cplx, M, N, K)[0] == rows[cplx], (cplx, M, N, K)
-    for cplx, M, N, K in [(1, 23, 11, 1 << 22), (0, 2, 2, 1 << 20), (0, 1, 8, 160000), (0, 31, 11, 567000)]:
+    for cplx, M, N, K in [(0, 2, 2, 1 << 20), (0, 1, 8, 160000), (0, 31, 11, 567000)]:
         assert tsm.choose(tsm.KIND_TSMM, cplx, M, N, K)[0] != rows[cplx], (cplx, M, N, K)
+    assert not cm.heuristic_pick(tsm.KIND_TSMM, 0, 36, 3, 1 << 23)[0].endswith("_row")
     lib = tsm.load()
     other = [v["index"] for v in tsm.variants(tsm.KIND_TSMM) if v["name"] == "tsmm_r64_rt_npt4_u2"][0]
     assert lib.tsm_set_tuning(tsm.KIND_TSMM, 0, 11, 6, 5000, other, 152) == 0
