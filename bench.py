@@ -883,7 +883,7 @@ def run_gs_extra(flatA, flatB, K, bw, p64):
     del Bw
     torch.cuda.empty_cache()
     return {"what": "tsm_gs_step: TSMTTSM (op C) then TSMM (alpha=-1, beta=1) on one stream, C on the device; "
-                    "small_k: the default path (fused for K <= 2^15), the two products, the fused kernel, and "
+                    "small_k: the default path (fused for the shortest), the two products, the fused kernel, and "
                     "each product alone",
             "roofline_pct_all": 100 * ideal / meas, "calls": out, "small_k": small}
 
