@@ -155,8 +155,10 @@ struct MmShape {
 
 size_t mm_smem(int M, int N, int cplx) { return (size_t)M * N * (cplx ? 2 : 1) * sizeof(double); }
 
+// The limit is set to the same value every time: one set to a launch's own
+// need could be lowered by another thread before that launch.
 cudaError_t allow_smem(const void* kernel, size_t smem) {
-    return smem > 48 * 1024 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+    return smem > 48 * 1024 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024)
                             : cudaSuccess;
 }
 
@@ -227,6 +229,8 @@ template <bool CPLX, bool GEN>
 cudaError_t launch_as(const TsmmArgs& a, const MmShape& s, int grid, int64_t rows, cudaStream_t st) {
     size_t smem = mm_smem(a.M, a.N, CPLX);
     const Kernel k = kernel_for<CPLX, GEN>(s.T);
+    cudaError_t e = allow_smem((const void*)k, smem);
+    if (e != cudaSuccess) return e;
     // Shared memory that leaves room for this grid's CTAs per SM and no more:
     // with CTAs of the neighbouring kernels waiting on some SMs, the placement
     // would else put two on one SM and none on another.  Complex 33 x 20, 1000
@@ -234,8 +238,7 @@ cudaError_t launch_as(const TsmmArgs& a, const MmShape& s, int grid, int64_t row
     const int sms = device_info().sm_count, cps = (grid + sms - 1) / sms;
     if (cps < resident_ctas((const void*)k, s.block, smem))
         smem = std::max<size_t>(smem, (size_t)228 * 1024 / (cps + 1) + 1024);
-    const cudaError_t e = allow_smem((const void*)k, smem);
-    if (e != cudaSuccess) return e;
+    if ((e = allow_smem((const void*)k, smem)) != cudaSuccess) return e;
     // the shortest start early at any grid: their CTAs are soon placed
     if ((double)a.M * a.N * (CPLX ? 4 : 1) * (double)a.K < 1e7)
         return launch_early(pdl_enabled(), k, grid, s.block, smem, st, a, s.tpr, s.L, rows);

@@ -252,7 +252,10 @@ cudaError_t launch_row(const TsmttsmArgs& a, int grid, cudaStream_t s) {
     if (cps < resident_ctas((const void*)k, r.block, 0)) {
         smem = limit_smem(cps);
         if (smem > 48 * 1024) {
-            const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            // (the largest value ever used: a limit of each launch's own could be
+            // lowered by another thread before the launch)
+            const cudaError_t e =
+                cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit_smem(1));
             if (e != cudaSuccess) return e;
         }
     }

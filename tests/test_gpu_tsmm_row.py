@@ -79,3 +79,36 @@ def test_rule(tsm):
     assert lib.tsm_set_tuning(tsm.KIND_TSMM, 0, 11, 6, 5000, other, 152) == 0
     assert tsm.choose(tsm.KIND_TSMM, 0, 11, 6, 5000) == (other, 152)
     assert tsm.choose(tsm.KIND_TSMM, 0, 11, 6, 20000)[0] == rows[0]
+
+
+def test_threads_with_different_shared_memory(tsm):
+    """Threads whose launches of one kernel pin different numbers of CTAs per
+    SM, and so ask for different amounts of shared memory, at the same time."""
+    import threading
+
+    import torch
+    shapes = [(16, 16, 500), (16, 16, 60000), (60, 60, 700), (60, 60, 30000)]
+    errors = []
+
+    def work(M, N, K):
+        try:
+            st = torch.cuda.Stream()
+            with torch.cuda.stream(st):
+                A = torch.randint(-3, 4, (K, M), device="cuda").to(torch.float64)
+                C = torch.randint(-3, 4, (M, N), device="cuda").to(torch.float64)
+                B, G = torch.empty((K, N), dtype=torch.float64, device="cuda"), torch.empty_like(C)
+                for _ in range(150):
+                    tsm.tsmm(A, C, B, 1.0, 0.0)
+                    tsm.tsmttsm(A, B, G)
+                st.synchronize()
+                if not (torch.equal(B, A @ C) and torch.equal(G, A.T @ B)):
+                    errors.append((M, N, K, "values"))
+        except Exception as e:
+            errors.append((M, N, K, repr(e)))
+
+    threads = [threading.Thread(target=work, args=s) for s in shapes]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
