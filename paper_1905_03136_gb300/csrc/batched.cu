@@ -772,6 +772,10 @@ tsm_status tsm_batched_create(const tsm_batch_desc* d, int count, tsm_batch** ou
         Inst& in = inst[i];
         const int first = (int)items.size();
         const int lg = (d[i].config >> 8) & 0xFF;
+        // a TSMM without rows has nothing to write, and its C (which an item
+        // would stage) may be null; a TSMTTSM without rows still applies beta,
+        // in one empty item
+        if (in.K == 0 && in.kind == TSM_KIND_TSMM) continue;
         auto cut = [&](int64_t from, int64_t to, int64_t rows) {
             do {
                 Item it;
@@ -820,7 +824,7 @@ tsm_status tsm_batched_create(const tsm_batch_desc* d, int count, tsm_batch** ou
     b->ctas = ctas;
     b->smem = smem;
     bool ok = cudaMalloc(&b->d_inst, sizeof(Inst) * count) == cudaSuccess &&
-              cudaMalloc(&b->d_items, sizeof(Item) * items.size()) == cudaSuccess &&
+              cudaMalloc(&b->d_items, sizeof(Item) * std::max<size_t>(items.size(), 1)) == cudaSuccess &&
               cudaMalloc(&b->d_counter, sizeof(unsigned)) == cudaSuccess &&
               cudaMalloc(&b->d_tickets, sizeof(unsigned) * std::max(n_tickets, 1)) == cudaSuccess &&
               cudaMalloc(&b->d_parts, sizeof(double) * std::max<int64_t>(part_doubles, 1)) == cudaSuccess;
