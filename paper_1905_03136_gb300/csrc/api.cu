@@ -48,6 +48,19 @@ std::map<std::pair<int, cudaStream_t>, Workspace*> g_ws;
 
 }  // namespace
 
+// Clears device memory before returning.  A memset on the legacy stream alone
+// would neither wait for nor hold back work on a non-blocking stream, and one
+// on the caller's stream would become part of a graph being captured there.
+cudaError_t zero_now(void* p, size_t bytes) {
+    cudaStream_t s = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return e;
+    e = cudaMemsetAsync(p, 0, bytes, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaStreamDestroy(s);
+    return e;
+}
+
 tsm_status workspace_get(cudaStream_t stream, size_t partial_bytes, int tickets, Workspace** out) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return TSM_ERR_NO_DEVICE;
@@ -82,7 +95,11 @@ tsm_status workspace_get(cudaStream_t stream, size_t partial_bytes, int tickets,
             w->tickets = nullptr;
             return TSM_ERR_ALLOC;
         }
-        if (cudaMemset(w->tickets, 0, sizeof(unsigned) * tc) != cudaSuccess) return TSM_ERR_LAUNCH;
+        if (zero_now(w->tickets, sizeof(unsigned) * tc) != cudaSuccess) {
+            w->partial_bytes = 0;  // the next call starts over
+            w->ticket_count = 0;
+            return TSM_ERR_LAUNCH;
+        }
         w->gs_gen = 0u;  // the barrier flag starts at zero again
         w->partial_bytes = pb;
         w->ticket_count = tc;

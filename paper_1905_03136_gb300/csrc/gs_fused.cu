@@ -406,11 +406,7 @@ tsm_status tsm_gs_status(tsm_stream_t stream) {
     unsigned err = 0;
     unsigned* p = ws->tickets + gsf::kErrWord;
     if (cudaMemcpy(&err, p, sizeof(unsigned), cudaMemcpyDeviceToHost) != cudaSuccess) return TSM_ERR_LAUNCH;
-    if (err) {
-        const unsigned zero = 0;
-        if (cudaMemcpy(p, &zero, sizeof(unsigned), cudaMemcpyHostToDevice) != cudaSuccess) return TSM_ERR_LAUNCH;
-        return TSM_ERR_TIMEOUT;
-    }
+    if (err) return zero_now(p, sizeof(unsigned)) == cudaSuccess ? TSM_ERR_TIMEOUT : TSM_ERR_LAUNCH;
     return TSM_OK;
 }
 

@@ -1302,11 +1302,7 @@ extern "C" tsm_status tsm_split_status(tsm_stream_t stream) {
     int err = 0;
     int* p = reinterpret_cast<int*>(ws->tickets) + split::kStatusWord;
     if (cudaMemcpy(&err, p, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return TSM_ERR_LAUNCH;
-    if (err) {
-        const int zero = 0;
-        if (cudaMemcpy(p, &zero, sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) return TSM_ERR_LAUNCH;
-        return TSM_ERR_TIMEOUT;
-    }
+    if (err) return zero_now(p, sizeof(int)) == cudaSuccess ? TSM_ERR_TIMEOUT : TSM_ERR_LAUNCH;
     return TSM_OK;
 }
 

@@ -172,6 +172,9 @@ struct Workspace {
 };
 tsm_status workspace_get(cudaStream_t stream, size_t partial_bytes, int tickets, Workspace** out);
 
+// Clears device memory before returning (api.cu).
+cudaError_t zero_now(void* p, size_t bytes);
+
 // The Gram-Schmidt step as one cooperative kernel (gs_fused.cu), and the
 // rule by which tsm_gs_step picks it over the two products.
 tsm_status gs_fused_run(tsm_dtype dtype, int M, int N, int64_t K, const void* A, int64_t lda, void* B,
