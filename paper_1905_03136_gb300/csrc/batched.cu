@@ -832,18 +832,24 @@ tsm_status tsm_batched_create(const tsm_batch_desc* d, int count, tsm_batch** ou
         tsm_batched_destroy(b);
         return TSM_ERR_ALLOC;
     }
-    if (cudaMemcpy(b->d_inst, inst.data(), sizeof(Inst) * count, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(b->d_items, items.data(), sizeof(Item) * items.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemset(b->d_tickets, 0, sizeof(unsigned) * std::max(n_tickets, 1)) != cudaSuccess) {
-        tsm_batched_destroy(b);
-        return TSM_ERR_LAUNCH;
-    }
-    // capture {counter reset, persistent kernel} once
     cudaStream_t cs;
     if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) {
         tsm_batched_destroy(b);
         return TSM_ERR_LAUNCH;
     }
+    // The plan is in place before this returns: the batch may run on any
+    // stream, and nothing would order a non-blocking one after copies and a
+    // memset on the legacy stream.
+    if (cudaMemcpyAsync(b->d_inst, inst.data(), sizeof(Inst) * count, cudaMemcpyHostToDevice, cs) != cudaSuccess ||
+        cudaMemcpyAsync(b->d_items, items.data(), sizeof(Item) * items.size(), cudaMemcpyHostToDevice, cs) !=
+            cudaSuccess ||
+        cudaMemsetAsync(b->d_tickets, 0, sizeof(unsigned) * std::max(n_tickets, 1), cs) != cudaSuccess ||
+        cudaStreamSynchronize(cs) != cudaSuccess) {
+        cudaStreamDestroy(cs);
+        tsm_batched_destroy(b);
+        return TSM_ERR_LAUNCH;
+    }
+    // capture {counter reset, persistent kernel} once
     bool cap = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
     if (cap) {
         cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned), cs);

@@ -61,3 +61,24 @@ def test_first_call_on_a_side_stream(tsm, path):
     side.synchronize()
     got = C.cpu()  # (waits for the default stream)
     assert torch.equal(got, want.cpu())
+
+
+def test_batch_made_while_the_default_stream_is_busy(tsm):
+    """A batch's plan (items, instances, tickets) is in place when create
+    returns: run on a side stream while the default stream has work queued."""
+    import torch
+    from paper_1905_03136_gb300 import batched
+    A = torch.randint(-3, 4, (30000, 5), device="cuda").to(torch.float64)
+    B = torch.randint(-3, 4, (30000, 3), device="cuda").to(torch.float64)
+    G = torch.full((5, 3), 7.0, dtype=torch.float64, device="cuda")
+    want = A.T @ B
+    descs = [batched.desc(batched.TSMTTSM, A, B, G, config=10 << 8)]
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for size in (256, 512, 1024, 4096):
+        _fill_free_memory(size, 16)
+    torch.cuda._sleep(1_000_000_000)
+    batch = batched.Batch(descs)
+    batch.run(stream=side)
+    side.synchronize()
+    assert torch.equal(G.cpu(), want.cpu())
