@@ -20,7 +20,9 @@
  * Ownership: the model owns its device buffers (parameters, gradients, Adam
  * moments, partial sums of the gradient); X (n x D row-major), targets and
  * outputs are caller-owned DEVICE float arrays.  Calls are asynchronous on
- * `stream` except the host<->device parameter copies, which synchronize.
+ * `stream` except the host<->device copies of parameters and gradients, which
+ * wait for every earlier call on the model, on whatever stream, and are done
+ * when they return (work replayed from a captured graph the caller waits for).
  * Every reduction over samples runs in an order fixed by n and the device,
  * so training is bitwise reproducible.  Errors: INVALID_VALUE for null
  * pointers, n < 1 or n > max_batch, D or H out of range.

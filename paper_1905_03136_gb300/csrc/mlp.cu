@@ -21,6 +21,9 @@
 #include <cstddef>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
+#include <new>
+#include <utility>
 #include <vector>
 
 #include "fp64_common.cuh"
@@ -38,6 +41,8 @@ struct tsm_mlp {
     int grid_max;   // CTAs the shares are sized for
     int stride;     // P rounded up to a multiple of four
     int64_t step;
+    mutable std::mutex mu;
+    mutable std::vector<std::pair<cudaStream_t, cudaEvent_t>> used;  // last work on each other stream than the legacy one
 };
 
 namespace tsm {
@@ -393,6 +398,38 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
     p[q] -= lr * (mq / c1) / (sqrtf(vq / c2) + eps);
 }
 
+// The host copies run on the legacy stream, which non-blocking streams do not
+// wait for, nor it for them.  note_use records where a stream's last work on
+// the model ends; the next copy has the legacy stream wait for all of them
+// and forgets them.  (Work being captured runs when its graph does: the
+// caller orders that.)
+cudaError_t note_use(tsm_mlp* m, cudaStream_t s) try {
+    if (s == nullptr || s == cudaStreamLegacy) return cudaSuccess;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(s, &st);
+    if (e != cudaSuccess || st != cudaStreamCaptureStatusNone) return e;
+    std::lock_guard<std::mutex> lock(m->mu);
+    for (const auto& u : m->used)
+        if (u.first == s) return cudaEventRecord(u.second, s);
+    m->used.reserve(m->used.size() + 1);
+    cudaEvent_t ev = nullptr;
+    if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess) return e;
+    m->used.emplace_back(s, ev);
+    return cudaEventRecord(ev, s);
+} catch (...) {
+    return cudaErrorMemoryAllocation;
+}
+cudaError_t join_uses(const tsm_mlp* m) {
+    std::lock_guard<std::mutex> lock(m->mu);
+    for (const auto& u : m->used) {
+        const cudaError_t e = cudaStreamWaitEvent(nullptr, u.second, 0);
+        if (e != cudaSuccess) return e;
+    }
+    for (const auto& u : m->used) cudaEventDestroy(u.second);
+    m->used.clear();
+    return cudaSuccess;
+}
+
 uint64_t splitmix(uint64_t& s) {
     uint64_t z = (s += 0x9E3779B97F4A7C15ull);
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
@@ -412,7 +449,7 @@ tsm_status tsm_mlp_create(int in_dim, int hidden, int max_batch, uint64_t seed, 
         max_batch < 1)
         return TSM_ERR_INVALID_VALUE;
     *out = nullptr;
-    tsm_mlp* m = (tsm_mlp*)calloc(1, sizeof(tsm_mlp));
+    tsm_mlp* m = new (std::nothrow) tsm_mlp();
     if (!m) return TSM_ERR_ALLOC;
     const mlp::Off o = mlp::offsets(in_dim, hidden);
     m->D = in_dim;
@@ -440,9 +477,17 @@ tsm_status tsm_mlp_create(int in_dim, int hidden, int max_batch, uint64_t seed, 
     for (int i = 0; i < hidden * in_dim; ++i) h[o.W1 + i] = uni(1.0f / sqrtf((float)in_dim));
     for (int i = 0; i < hidden * hidden; ++i) h[o.W2 + i] = uni(1.0f / sqrtf((float)hidden));
     for (int i = 0; i < hidden; ++i) h[o.w3 + i] = uni(1.0f / sqrtf((float)hidden));
-    if (cudaMemcpy(m->params, h.data(), pb, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemset(m->grads, 0, pb) != cudaSuccess || cudaMemset(m->m, 0, pb) != cudaSuccess ||
-        cudaMemset(m->v, 0, pb) != cudaSuccess) {
+    // in place before this returns, whatever stream the model is used on
+    cudaStream_t cs = nullptr;
+    ok = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess;
+    if (ok) {
+        ok = cudaMemcpyAsync(m->params, h.data(), pb, cudaMemcpyHostToDevice, cs) == cudaSuccess &&
+             cudaMemsetAsync(m->grads, 0, pb, cs) == cudaSuccess && cudaMemsetAsync(m->m, 0, pb, cs) == cudaSuccess &&
+             cudaMemsetAsync(m->v, 0, pb, cs) == cudaSuccess;
+        ok = cudaStreamSynchronize(cs) == cudaSuccess && ok;
+        cudaStreamDestroy(cs);
+    }
+    if (!ok) {
         tsm_mlp_destroy(m);
         return TSM_ERR_LAUNCH;
     }
@@ -458,18 +503,20 @@ void tsm_mlp_destroy(tsm_mlp* m) {
     cudaFree(m->v);
     cudaFree(m->parts);
     cudaFree(m->lparts);
-    free(m);
+    for (const auto& u : m->used) cudaEventDestroy(u.second);
+    delete m;
 }
 
 int tsm_mlp_param_count(const tsm_mlp* m) { return m ? m->P : -1; }
 
 tsm_status tsm_mlp_set_params(tsm_mlp* m, const float* host) {
     if (!m || !host) return TSM_ERR_INVALID_VALUE;
+    if (mlp::join_uses(m) != cudaSuccess) return TSM_ERR_LAUNCH;
     if (cudaMemcpy(m->params, host, sizeof(float) * m->P, cudaMemcpyHostToDevice) != cudaSuccess)
         return TSM_ERR_LAUNCH;
     // a new parameter vector restarts the optimiser
     if (cudaMemset(m->m, 0, sizeof(float) * m->P) != cudaSuccess ||
-        cudaMemset(m->v, 0, sizeof(float) * m->P) != cudaSuccess)
+        cudaMemset(m->v, 0, sizeof(float) * m->P) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess)
         return TSM_ERR_LAUNCH;
     m->step = 0;
     return TSM_OK;
@@ -477,6 +524,7 @@ tsm_status tsm_mlp_set_params(tsm_mlp* m, const float* host) {
 
 tsm_status tsm_mlp_get_params(const tsm_mlp* m, float* host) {
     if (!m || !host) return TSM_ERR_INVALID_VALUE;
+    if (mlp::join_uses(m) != cudaSuccess) return TSM_ERR_LAUNCH;
     return cudaMemcpy(host, m->params, sizeof(float) * m->P, cudaMemcpyDeviceToHost) == cudaSuccess
                ? TSM_OK
                : TSM_ERR_LAUNCH;
@@ -484,6 +532,7 @@ tsm_status tsm_mlp_get_params(const tsm_mlp* m, float* host) {
 
 tsm_status tsm_mlp_get_grads(const tsm_mlp* m, float* host) {
     if (!m || !host) return TSM_ERR_INVALID_VALUE;
+    if (mlp::join_uses(m) != cudaSuccess) return TSM_ERR_LAUNCH;
     return cudaMemcpy(host, m->grads, sizeof(float) * m->P, cudaMemcpyDeviceToHost) == cudaSuccess
                ? TSM_OK
                : TSM_ERR_LAUNCH;
@@ -498,7 +547,8 @@ tsm_status tsm_mlp_forward(tsm_mlp* m, const float* X, int n, float* y, tsm_stre
     const int tiles = (n - 1) / mlp::TS + 1;
     mlp::k_mlp<false><<<std::min(tiles, m->grid_max), mlp::kThreads, smem, (cudaStream_t)stream>>>(
         m->params, m->D, m->H, X, nullptr, n, y, nullptr, 0, nullptr);
-    return cudaGetLastError() == cudaSuccess ? TSM_OK : TSM_ERR_LAUNCH;
+    if (cudaGetLastError() != cudaSuccess) return TSM_ERR_LAUNCH;
+    return mlp::note_use(m, (cudaStream_t)stream) == cudaSuccess ? TSM_OK : TSM_ERR_LAUNCH;
 }
 
 tsm_status tsm_mlp_backward(tsm_mlp* m, const float* X, const float* t, int n, float* loss,
@@ -513,10 +563,10 @@ tsm_status tsm_mlp_backward(tsm_mlp* m, const float* X, const float* t, int n, f
                                                        m->lparts);
     if (cudaGetLastError() != cudaSuccess) return TSM_ERR_LAUNCH;
     const int quads = (m->P + 4 * mlp::kQuads - 1) / (4 * mlp::kQuads);
-    return launch_early(pdl_enabled(), mlp::k_mlp_sum, quads + 1, mlp::kSlices * mlp::kQuads, 0, s, m->parts,
-                        m->stride, m->lparts, grid, m->P, n, m->grads, loss) == cudaSuccess
-               ? TSM_OK
-               : TSM_ERR_LAUNCH;
+    if (launch_early(pdl_enabled(), mlp::k_mlp_sum, quads + 1, mlp::kSlices * mlp::kQuads, 0, s, m->parts, m->stride,
+                     m->lparts, grid, m->P, n, m->grads, loss) != cudaSuccess)
+        return TSM_ERR_LAUNCH;
+    return mlp::note_use(m, s) == cudaSuccess ? TSM_OK : TSM_ERR_LAUNCH;
 }
 
 tsm_status tsm_mlp_adam(tsm_mlp* m, float lr, float beta1, float beta2, float eps, tsm_stream_t stream) {
@@ -528,7 +578,8 @@ tsm_status tsm_mlp_adam(tsm_mlp* m, float lr, float beta1, float beta2, float ep
     const float c2 = 1.0f - powf(beta2, (float)m->step);
     mlp::k_adam<<<(m->P + 127) / 128, 128, 0, (cudaStream_t)stream>>>(m->params, m->grads, m->m, m->v, m->P, lr,
                                                                       beta1, beta2, eps, c1, c2);
-    return cudaGetLastError() == cudaSuccess ? TSM_OK : TSM_ERR_LAUNCH;
+    if (cudaGetLastError() != cudaSuccess) return TSM_ERR_LAUNCH;
+    return mlp::note_use(m, (cudaStream_t)stream) == cudaSuccess ? TSM_OK : TSM_ERR_LAUNCH;
 }
 
 }  // extern "C"
