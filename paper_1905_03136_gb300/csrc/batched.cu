@@ -712,8 +712,10 @@ tsm_status tsm_batched_create(const tsm_batch_desc* d, int count, tsm_batch** ou
     for (int i = 0; i < count; ++i)
         if (d[i].kind == TSM_KIND_TSMM)
             smem = std::max(smem, (size_t)d[i].M * d[i].N * (d[i].dtype == TSM_C64 ? 2 : 1) * sizeof(double));
+    // The limit is the kernel function's, not the plan's: always the largest C,
+    // since a later plan's own need would lower it under an earlier one.
     if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(k_batched, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        cudaFuncSetAttribute(k_batched, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxStagedC) != cudaSuccess)
         return TSM_ERR_LAUNCH;
     int occ = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batched, kThreads, smem) != cudaSuccess || occ < 1)

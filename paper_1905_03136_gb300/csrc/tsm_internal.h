@@ -87,6 +87,9 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t sme
     return launch_early(pdl_allowed((const void*)kernel, grid, block, smem), kernel, grid, block, smem, s, args...);
 }
 
+// Bytes of the largest C that a kernel stages in shared memory (complex 64 x 64).
+constexpr int kMaxStagedC = 64 * 64 * 2 * (int)sizeof(double);
+
 typedef cudaError_t (*TsmttsmLaunch)(const TsmttsmArgs&, int grid, cudaStream_t);
 typedef cudaError_t (*TsmmLaunch)(const TsmmArgs&, int grid, cudaStream_t);
 // Resident CTAs per SM for this variant and shape (0 if it cannot run).
