@@ -325,7 +325,7 @@ tsm_status run(tsm_dtype dtype, int M, int N, int64_t K, const void* A, int64_t 
     const Kernel k = kernel_for(tile_for(M, N), cplx);
     const size_t smem = smem_for(M, N, cplx);
     if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxStagedC) != cudaSuccess)
         return TSM_ERR_LAUNCH;
     int occ = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kThreads, smem) != cudaSuccess || occ < 1)

@@ -135,7 +135,7 @@ cudaError_t launch_tsmm_as(const TsmmArgs& a, int grid, cudaStream_t s) {
     const size_t smem = tsmm_smem<TPR, NPT, U, CPLX>(a.M, a.N);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_tsmm<TPR, NPT, U, CPLX, GEN>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxStagedC);
         if (e != cudaSuccess) return e;
     }
     return launch_pdl(k_tsmm<TPR, NPT, U, CPLX, GEN>, grid, kBlock, smem, s, a);
@@ -153,7 +153,7 @@ int occ_tsmm(int M, int N) {
     const size_t smem = tsmm_smem<TPR, NPT, U, CPLX>(M, N);
     if (smem > 48 * 1024 &&
         cudaFuncSetAttribute(k_tsmm<TPR, NPT, U, CPLX, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess)
+                             kMaxStagedC) != cudaSuccess)
         return 0;
     int n = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_tsmm<TPR, NPT, U, CPLX, false>, kBlock, smem) !=

@@ -146,7 +146,7 @@ cudaError_t launch_tsmm_rt_as(const TsmmArgs& a, int grid, cudaStream_t s) {
     const size_t smem = (size_t)a.M * a.N * (CPLX ? 2 : 1) * sizeof(double);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_tsmm_rt<NPT, U, CPLX, GEN>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxStagedC);
         if (e != cudaSuccess) return e;
     }
     return launch_pdl(k_tsmm_rt<NPT, U, CPLX, GEN>, grid, kBlock, smem, s, a, tpr);
@@ -162,8 +162,8 @@ template <int NPT, int U, bool CPLX>
 int occ_tsmm_rt(int M, int N) {
     const size_t smem = (size_t)M * N * (CPLX ? 2 : 1) * sizeof(double);
     if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(k_tsmm_rt<NPT, U, CPLX, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-            cudaSuccess)
+        cudaFuncSetAttribute(k_tsmm_rt<NPT, U, CPLX, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kMaxStagedC) != cudaSuccess)
         return 0;
     int n = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_tsmm_rt<NPT, U, CPLX, false>, kBlock, smem) != cudaSuccess)

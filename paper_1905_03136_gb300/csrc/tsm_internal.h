@@ -87,7 +87,10 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t sme
     return launch_early(pdl_allowed((const void*)kernel, grid, block, smem), kernel, grid, block, smem, s, args...);
 }
 
-// Bytes of the largest C that a kernel stages in shared memory (complex 64 x 64).
+// Bytes of the largest C that a kernel stages in shared memory (complex
+// 64 x 64).  Kernels that stage C above 48 KB set their limit to this: it is
+// state of the kernel function, and one set to a launch's own need could be
+// lowered by another thread before that launch.
 constexpr int kMaxStagedC = 64 * 64 * 2 * (int)sizeof(double);
 
 typedef cudaError_t (*TsmttsmLaunch)(const TsmttsmArgs&, int grid, cudaStream_t);
