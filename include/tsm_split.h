@@ -15,16 +15,23 @@
  * are recombined and reduced over K in binary64.  Complex data is handled
  * as the real product of the interleaved (re, im) columns.
  *
- * Accuracy: with S slices each input keeps 8S - 1 bits below its column's
- * running maximum and slice products of combined weight below 2^-(8S+6)
- * are dropped, so |C_split - C_exact| is a few units of 2^-(8S-1) relative
- * to sum |a||b| per entry.  S = 6 (tsm_tsmttsm_split): normwise relative
- * error against the FP64 oracle about 1e-14 on uniform and log-uniform
- * inputs, within the 1e-12 bar of the FP64 path; S = 5: about 4e-12;
- * S = 4: about 1e-9 (fewer tensor-core products, fewer accumulator
- * columns, faster).  Inputs that are small integers (or any values with at
- * most 8S - 1 significant bits below the column maximum) give the exact
- * result.  Inputs must be finite (NaN/Inf are not propagated; use
+ * Accuracy: K is cut into ranges (fixed by the shape and the device), within
+ * which every column has an exponent e that follows the largest magnitude
+ * met so far, in steps of 16 rows: 2^e bounds it, except that with S = 5 and
+ * 6 e is at most one higher in a range's first 128 rows, and a value may
+ * exceed 2^e by less than a bit a few times before e follows.  Inputs keep
+ * 8S - 1 bits below 2^e, rounded (S = 4: truncated), and slice products of
+ * combined weight below 2^-(8S+6) are dropped.  |C_split - C_exact| of an
+ * entry is a few units of 2^-(8S-1) relative to the sum over the rows of
+ * the product of the two columns' running maxima: rows that follow much
+ * larger ones of their column lose the bits below them, rows before those
+ * keep theirs.  Normwise relative error against the FP64 oracle on uniform,
+ * normal and log-uniform inputs of 10^3 to 4 10^6 rows: S = 6
+ * (tsm_tsmttsm_split) 8e-15 to 1.3e-13, within the 1e-12 bar of the FP64
+ * path; S = 5 1e-12 to 4e-11; S = 4 about 1e-9 (fewer tensor-core
+ * products, fewer accumulator columns, faster).  Inputs that are small
+ * integers (products and sums exact in the bits kept) give the exact result.
+ * Inputs must be finite (NaN/Inf are not propagated; use
  * tsm_tsmttsm for them).  Results are deterministic for a fixed problem,
  * slice count and device.
  *

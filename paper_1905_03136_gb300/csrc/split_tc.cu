@@ -359,9 +359,10 @@ static_assert(M_SEQ + 4 * MAX_GROUPS <= M_ABORT && M_TILE_INFO + 4 <= (int)kMisc
 // and the exponents are the plain running maxima of their range: any other
 // choice moves the results by as much as their error.  With 5 and 6 slices
 // digits are rounded, the exponents start from a scan of the range's first
-// rows, and a column may exceed its 2^e a few times; the error against 64
-// bits over 60 shapes of 10^3 .. 6 10^4 rows is 0.81 of that of truncated
-// digits and running maxima (geometric mean).
+// rows (at most a bit above the first step's), and a column may exceed its
+// 2^e a few times; the error against 64 bits over 60 shapes of 10^3 .. 6 10^4
+// rows, eight inputs each, is 0.78 of that of truncated digits and running
+// maxima in the geometric mean, 1.05 at most.
 template <int S>
 constexpr bool plain_digits() {
     return S == 4;
@@ -618,12 +619,17 @@ __global__ void __launch_bounds__(kThreadsPerSM, 1) k_split(const Params prm) {
         };
         double v[R];
         // The column exponents of a range start at the maximum over its
-        // first PRE_STEPS steps.  Without this every new maximum of a
-        // column's first rows ends an accumulation tile (normal data, 64 x
-        // 64 complex: 11.7 ms against 6.0 ms for uniform data, whose
-        // exponents settle at once).
+        // first PRE_STEPS steps, if that is at most a bit above the first
+        // step's: rounding then costs the first rows no more than truncation
+        // at the running maximum did.  Columns that grow faster start at the
+        // first step's, so that small rows before large ones keep their
+        // bits.  Without the scan every new maximum of a column's first rows
+        // ends an accumulation tile, at about 10 us of the CTA (normal data:
+        // real 24 x 40, S = 5, 10^6 rows 569 us against 352, complex 64 x 64,
+        // 10^5 rows 404 against 191).
         const int srange = (int)min(prm.steps_per_range, (int64_t)nsteps + 1);
         if (!plain_digits<S>()) {
+            int* first = exps;  // not in use yet: the ranges' first steps' exponents [MAX_RANGES][NE], ndig >= MAX_RANGES
             for (int j = 0; j < MAX_RANGES && j * srange < nsteps; ++j) {
                 const int pre = min(min(nsteps - j * srange, srange), PRE_STEPS) * ncg;
                 for (int u = warp; u < pre; u += NCONV_WARPS) {
@@ -632,9 +638,16 @@ __global__ void __launch_bounds__(kThreadsPerSM, 1) k_split(const Params prm) {
                     const uint32_t hm = high_max(v);
                     if (slot < P + Qw && g == 0) {
                         atomicMax(&col_e0[j * NE + slot], exp_from_hi(hm));
-                        if (j == 0) atomicMax(&col_e[slot], exp_from_hi(hm));
+                        if (u < ncg) first[j * NE + slot] = exp_from_hi(hm);
                     }
                 }
+            }
+            asm volatile("bar.sync 1, %0;" ::"r"(NCONV_WARPS * 32) : "memory");
+#pragma unroll 1
+            for (int i = threadIdx.x; i < MAX_RANGES * NE; i += NCONV_WARPS * 32) {
+                int e = col_e0[i];
+                if (e > first[i] + 1) col_e0[i] = e = first[i];
+                if (i < NE) col_e[i] = e;
             }
             asm volatile("bar.sync 1, %0;" ::"r"(NCONV_WARPS * 32) : "memory");
         }
