@@ -613,7 +613,7 @@ tsm_status run_tsmttsm(tsm_op opA, tsm_dtype dtype, int M, int N, int64_t K, con
     std::lock_guard<std::mutex> lock(pdl_mutex());
     a.early = pdl_early(stream, in, 2);
     if (var.tsmttsm(a, g, stream) != cudaSuccess) return TSM_ERR_LAUNCH;
-    if (a.final_pass && launch_tsmttsm_final(a, g, cplx, stream) != cudaSuccess) return TSM_ERR_LAUNCH;
+    if (a.final_pass && launch_tsmttsm_final(a, g, cplx, var.final_pass, stream) != cudaSuccess) return TSM_ERR_LAUNCH;
     pdl_note(stream, operand_range(C, M, ldc, N, cplx), a.early);
     return TSM_OK;
 }

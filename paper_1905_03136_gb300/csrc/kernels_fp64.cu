@@ -262,11 +262,15 @@ namespace {
 // lane takes a few dozen partials, the pass is a handful of L2 round trips
 // however many CTAs wrote partials.  Small CTAs spread those over more SMs:
 // complex 8 x 8, 10^5 rows 55.3 us a call with CTAs of 256 threads, 53.2 with
-// 64.  Behind a short product the launch may start early whatever its size,
-// its few CTAs only wait (complex 8 x 8, 3000 rows: 11 us a call, 14 without);
-// behind a long one that lets the product after it start too soon, on SMs
-// that free up unevenly (the Gram-Schmidt step of complex 60 x 4, 10^6 rows,
-// 3.29 ms instead of 3.16).
+// 64.  Behind a short product of a row kernel the launch may start early
+// whatever its size, its few CTAs only wait (complex 8 x 8, 3000 rows: 11 us a
+// call, 14 without); behind a long one that lets the product after it start
+// too soon, on SMs that free up unevenly (the Gram-Schmidt step of complex
+// 60 x 4, 10^6 rows, 3.29 ms instead of 3.16).  Behind the other kernels it
+// waits its turn: those that end in this pass have wide results, hundreds of
+// CTAs here, whose waiting took the SMs from the next product (complex
+// 64 x 60, 300 rows 32.9 us a call early, 26.9 not; real 64 x 64, 20000 rows
+// 155.9 and 150.5).
 constexpr int kFinalBlock = 64;
 template <int CC>
 __global__ void __launch_bounds__(kFinalBlock) k_tsmttsm_final(const TsmttsmArgs a, int G, int S) {
@@ -290,8 +294,8 @@ __global__ void __launch_bounds__(kFinalBlock) k_tsmttsm_final(const TsmttsmArgs
 
 }  // namespace
 
-cudaError_t launch_tsmttsm_final(const TsmttsmArgs& a, int grid, int cplx, cudaStream_t s) {
-    const bool early = short_product(a.M, a.N, a.K, cplx) && pdl_enabled();
+cudaError_t launch_tsmttsm_final(const TsmttsmArgs& a, int grid, int cplx, bool row, cudaStream_t s) {
+    const bool early = row && short_product(a.M, a.N, a.K, cplx) && pdl_enabled();
     const int MN = a.M * a.N;
     int S = 1;
     while (S < 32 && grid >= 16 * S) S *= 2;  // at least 8 partials per lane

@@ -114,7 +114,7 @@ extern "C" tsm_status tsm_tsmttsm_noalloc(tsm_op opA, tsm_dtype dtype, int M, in
     std::lock_guard<std::mutex> lock(pdl_mutex());
     a.early = 0;
     if (var->tsmttsm(a, grid, s) != cudaSuccess) return TSM_ERR_LAUNCH;
-    if (a.final_pass && launch_tsmttsm_final(a, grid, cplx, s) != cudaSuccess) return TSM_ERR_LAUNCH;
+    if (a.final_pass && launch_tsmttsm_final(a, grid, cplx, var->final_pass, s) != cudaSuccess) return TSM_ERR_LAUNCH;
     pdl_note(s, operand_range(C, M, ldc, N, cplx), 0);
     return TSM_OK;
 }

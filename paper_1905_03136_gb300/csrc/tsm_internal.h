@@ -132,7 +132,8 @@ constexpr int kFinalThreshold = 32768;
 inline bool short_product(int M, int N, int64_t K, int cplx) {
     return (double)M * N * (cplx ? 4 : 1) * (double)K <= 1e8;
 }
-cudaError_t launch_tsmttsm_final(const TsmttsmArgs& a, int grid, int cplx, cudaStream_t s);
+// (`row`: behind a row kernel)
+cudaError_t launch_tsmttsm_final(const TsmttsmArgs& a, int grid, int cplx, bool row, cudaStream_t s);
 
 // Index-independent part of the row kernel's rule (kernels_row.cu): the FP64
 // slots its tile takes per useful FMA, 0 if it cannot run the shape.
