@@ -379,9 +379,10 @@ static double tile_slots(const tsm_variant_info& f, int M, int N) {
 //     200000 rows 880 / 788; real 9 x 41, 10^6 rows 671 / 690 (1.04, 1.03: stays).
 //   from 2^21 rows on only where a loaded table has no entry of the shape (an
 //     empty table's plain heuristic is what the cost model is judged against),
-//     by the slots and by what the other's tile takes at no waste: complex
+//     by the slots and by what either kernel takes at no waste: complex
 //     45 x 32, 1.6 10^7 rows 1.20 times as fast, real 58 x 13 1.20, real 7 x 5
-//     1.22, complex 53 x 11 1.14; real 41 x 9 0.95, complex 50 x 13 0.95.
+//     1.22, complex 53 x 11 1.14; complex 50 x 13 (21 warps an SM) would be 0.95,
+//     real 11 x 23 0.96, complex 9 x 7 0.97: they stay.
 static bool row_preferred(const tsm_variant_info& other, int distance, int dtype, int M, int N, int64_t K) {
     const double slots = row_slots(M, N, dtype == TSM_C64);
     if (slots <= 0.0) return false;
@@ -396,8 +397,7 @@ static bool row_preferred(const tsm_variant_info& other, int distance, int dtype
         const int area = other.tile_m * other.tile_n;
         const bool cplx = dtype == TSM_C64;
         const double theirs = cplx ? (area == 1 ? 1.08 : 1.05) : area == 1 ? 1.25 : area < 16 ? 1.09 : 1.05;
-        const double own = cplx ? 1.05 : row_block(M, N, 0) <= 192 ? 1.2 : 1.09;
-        return waste * theirs > 1.04 * slots * own;
+        return waste * theirs > (cplx ? 1.05 : 1.04) * slots * row_long_cost(M, N, cplx);
     }
     if (narrow && fma < 5e5) return false;
     if (per_row < 64.0 && small_tile && waste < 1.3)

@@ -20,6 +20,7 @@
 // Every order is fixed by the shape and the grid, so results repeat bit for
 // bit.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -216,11 +217,15 @@ Kernel kernel_of(bool conj) {
 
 // Rows per register set: a few for the shortest strips, else one.
 template <bool CPLX>
+constexpr int rows_per_set(int T) {
+    return T == 1 ? (CPLX ? 2 : 4) : (T <= 3 && !CPLX ? 2 : 1);
+}
+template <bool CPLX>
 Kernel kernel_for(int T, bool conj) {
     switch (T) {
-        case 1: return kernel_of<1, CPLX ? 2 : 4, CPLX>(conj);
-        case 2: return kernel_of<2, CPLX ? 1 : 2, CPLX>(conj);
-        case 3: return kernel_of<3, CPLX ? 1 : 2, CPLX>(conj);
+        case 1: return kernel_of<1, rows_per_set<CPLX>(1), CPLX>(conj);
+        case 2: return kernel_of<2, rows_per_set<CPLX>(2), CPLX>(conj);
+        case 3: return kernel_of<3, rows_per_set<CPLX>(3), CPLX>(conj);
         case 4: return kernel_of<4, 1, CPLX>(conj);
         case 5: return kernel_of<5, 1, CPLX>(conj);
         case 6: return kernel_of<6, 1, CPLX>(conj);
@@ -234,6 +239,22 @@ Kernel kernel_for(int T, bool conj) {
         case 10: return kernel_of<10, 1, false>(false);
         default: return kernel_of<13, 1, false>(false);
     }
+}
+
+// Registers a thread, in the units they are handed out in (0: unknown).
+template <bool CPLX>
+int registers(int T) {
+    static std::atomic<int> known[16];
+    int r = known[T].load(std::memory_order_relaxed);
+    if (!r) {
+        cudaFuncAttributes at;
+        if (cudaFuncGetAttributes(&at, (const void*)kernel_for<CPLX>(T, false)) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        known[T].store(r = (at.numRegs + 7) / 8 * 8, std::memory_order_relaxed);
+    }
+    return r;
 }
 
 double row_work(int M, int N, int64_t K, int cplx) { return (double)K * M * N * (cplx ? 4 : 1); }
@@ -274,6 +295,19 @@ int occ_row(int M, int N) {
 // CTAs per SM by the work: one below 6 10^6 FMAs (3 10^6 if a CTA has no more
 // than six warps to hide its loads with), or where two would leave a CTA of
 // more fewer than 64 rows for its partial; two below 10^8; else what fits.
+// Three cases in the middle differ:
+//   two CTAs that fill the register file leave no room for the CTAs of the
+//     neighbours that wait on the SM, and some start a wave late (complex strips
+//     of 6 and 7 in CTAs of 256): one.  Complex 2 x 12, 78231 rows 27.9 / 20.0 us
+//     (two / one), 56 x 1, 40972 rows 29.0 / 23.3;
+//   real CTAs of more than ten warps with strips of five and more hold an SM's
+//     FMAs alone, up to 5 10^7 and 60000 rows: real 35 x 35, 19610 rows 56.8 / 44.2,
+//     48 x 11, 36707 rows 45.6 / 35.1, 24 x 29, 25177 rows 32.7 / 32.8, but 5 x 59,
+//     68213 rows 35.7 / 39.2;
+//   operands that do not fit L2 (129 MB) wait for DRAM, which real CTAs with
+//     fewer than 1200 FMAs per set of rows do not cover: three.  Real 64 x 2, 334665
+//     rows 103 / 83 (two / three), 8 x 8, 902858 rows 137 / 111, 17 x 10, 446205
+//     rows 234 / 170; with more FMAs real 32 x 5, 398825 rows 114 / 120.
 // Measured (us, one / two / what fits): real 6 x 6 at 50000 rows 9.1 / 10.6 /
 // 16.7, complex 50 x 50 at 5000 rows 99.6 / 108 / 99.6, real 22 x 22 at 52291
 // rows 80.6 / 52.7 / 60.6, complex 17 x 33 at 200000 rows 1211 / 849 / 788;
@@ -287,10 +321,19 @@ int grid_row(int M, int N, int64_t K) {
     const double fma = row_work(M, N, K, CPLX);
     int cps = occ;
     const bool few_warps = row_shape(M, N, CPLX).block <= 192;
-    if (fma < (few_warps ? 3e6 : 6e6) || (!few_warps && K < 128 * (int64_t)sms))
+    if (fma < (few_warps ? 3e6 : 6e6) || (!few_warps && K < 128 * (int64_t)sms)) {
         cps = 1;
-    else if (fma < 1e8)
-        cps = 2;
+    } else if (fma < 1e8) {
+        const RowShape& r = row_shape(M, N, CPLX);
+        const int set = r.block * r.T * rows_per_set<CPLX>(r.T);
+        const double bytes = 8.0 * (CPLX ? 2 : 1) * (M + N) * (double)K;
+        // (a waiting CTA of the final kernel: 64 threads of 48 registers at most)
+        const bool room = 2 * r.block * registers<CPLX>(r.T) + 64 * 48 <= 65536;
+        if (!room || (!CPLX && r.T >= 5 && r.block > 320 && fma < 5e7 && K < 60000))
+            cps = 1;
+        else
+            cps = !CPLX && set < 1200 && bytes > 9.5e7 ? 3 : 2;
+    }
     return sms * std::min(cps, occ);
 }
 
@@ -323,7 +366,15 @@ Variant make_row() {
 }  // namespace
 
 double row_slots(int M, int N, int cplx) { return row_shape(M, N, cplx).slots; }
-int row_block(int M, int N, int cplx) { return row_shape(M, N, cplx).block; }
+double row_long_cost(int M, int N, int cplx) {
+    const RowShape& r = row_shape(M, N, cplx);
+    if (!cplx) return r.block <= 192 || r.T == 1 ? 1.2 : 1.09;
+    if (r.T > 3) return 1.05;
+    // short strips leave the pipe idle where the SM's four schedulers do not
+    // have equally many warps
+    const int warps = r.block / 32 * std::max(occ_row<true>(M, N), 1);
+    return std::max(1.05, (warps + 3) / 4 * 4.0 / warps);
+}
 
 void register_row_variants(std::vector<Variant>& tsmttsm) {
     tsmttsm.push_back(make_row<false>());

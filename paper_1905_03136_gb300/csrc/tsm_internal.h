@@ -138,7 +138,7 @@ cudaError_t launch_tsmttsm_final(const TsmttsmArgs& a, int grid, int cplx, bool 
 // Index-independent part of the row kernel's rule (kernels_row.cu): the FP64
 // slots its tile takes per useful FMA, 0 if it cannot run the shape.
 double row_slots(int M, int N, int cplx);
-int row_block(int M, int N, int cplx);  // its CTA size
+double row_long_cost(int M, int N, int cplx);  // time over slots of a long product
 
 // Per-launch choice of the runtime-threads-per-row TSMM variants (kernels_rt.cu).
 void rt_tsmm_tpr(int N, int nptmax, int* tpr, int* npt);
