@@ -368,7 +368,7 @@ Variant make_row() {
 double row_slots(int M, int N, int cplx) { return row_shape(M, N, cplx).slots; }
 double row_long_cost(int M, int N, int cplx) {
     const RowShape& r = row_shape(M, N, cplx);
-    if (!cplx) return r.block <= 192 || r.T == 1 ? 1.2 : 1.09;
+    if (!cplx) return r.T == 1 ? 1.3 : r.block <= 192 ? 1.2 : 1.09;
     if (r.T > 3) return 1.05;
     // short strips leave the pipe idle where the SM's four schedulers do not
     // have equally many warps
