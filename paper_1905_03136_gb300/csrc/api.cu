@@ -449,11 +449,14 @@ static double stride_cost(const tsm_variant_info& f, int cplx, int N, int64_t K,
 //     8.1; real 1 x 8, 164000 rows 4.4 / 12.3.
 //   real 1 x 35, 1.6 10^7 rows (one result per thread): 1.59 times as fast; real
 //     6 x 47, 8 10^6 rows 1.13; real 36 x 3, 10^7 rows 2735 / 1890.
-//   Over 119 products from 2^22 rows on that the two rules take: 1.144 times as
-//     fast in the geometric mean, the worst 0.95.
-// Of 1982 drawn products below 2^22 rows the rule takes 1276, in the geometric mean 1.64 times
-// as fast there, four of them 3 to 7 % slower.
-static bool mm_preferred(const tsm_variant_info& other, int grid, int distance, int dtype, int M, int N, int64_t K) {
+//   where the other stays: real 2 x 23, 200000 rows 0.89 times as fast, real
+//     2 x 39, 8.9 10^6 rows, update 1777 / 1995, real 32 x 1, 5 10^6 rows 526 / 587,
+//     real 2 x 4, 10800 rows 2.1 / 2.5.
+// Of 1982 drawn products below 2^22 rows the rule takes 1310, in the geometric
+// mean 1.64 times as fast there, five of them 3 to 7 % slower (short complex
+// ones, the worst 8 x 10 with 30929 rows).
+static bool mm_preferred(const tsm_variant_info& other, int grid, int distance, int dtype, int M, int N, int64_t K,
+                         bool beta) {
     if (K >= ((int64_t)1 << 22) && distance == -2) return false;
     const int cplx = dtype == TSM_C64;
     const double per_row = (double)M * N * (cplx ? 4 : 1), fma = per_row * (double)K;
@@ -462,16 +465,25 @@ static bool mm_preferred(const tsm_variant_info& other, int grid, int distance, 
     // how much dearer the other has to be: the row kernel's own cost spreads
     // more at few columns of A and with short products
     const bool plain_rt = other.runtime_tile && npt < 3 && fma >= 3e7;
-    const double margin = M < 8 ? (plain_rt ? 1.04 : 1.15) : cplx ? (fma < 3e7 ? 1.04 : 1.015) : (fma < 3e7 ? 1.12 : 1.04);
+    const double margin = M < 8 ? (plain_rt ? 1.04 : 1.15)
+                          : cplx ? (fma < 3e7 ? 1.04 : 1.015)
+                                 : (fma < 3e7 ? 1.12 : 1.04);
     auto cheaper = [&] { return stride_cost(other, cplx, N, K, grid) > margin * mm_cost(M, N, K, cplx); };
     const bool slow_split = other.runtime_tile && !cplx && npt == 3;
     if (other.generated && M * N <= 4) return false;
     // single columns: the other kernels' threads each read a row on their own
-    if (N == 1 && M >= 16) return M >= (fma <= 1e8 ? 24 : 32) || fma <= 3e7;
+    if (N == 1 && M >= 16) return M >= (fma <= 1e8 ? 24 : 33) || fma <= 3e7;
     if (N == 1 && M >= 12) return fma <= 2.5e6;
     // one to three columns of A, and results that the runtime variant gives a
-    // thread each: its loads of A bound it
-    if (M < 4 && !cplx && other.runtime_tile && N >= 16 && fma > 5e6 && (npt == 1 || (npt == 3 && M > 1))) return true;
+    // thread each: its loads of A bound it, unless they come from L2; with
+    // three each, and B read as well, two columns are bound by memory
+    if (M < 4 && !cplx && other.runtime_tile && N >= 16 && fma > 5e6 && (npt == 1 || (npt == 3 && M > 1))) {
+        if (npt == 1 && M > 1 && !beta && 8.0 * (M + N) * (double)K < 9.5e7) return false;
+        return !(npt == 3 && M == 2 && beta && 8.0 * (M + 2 * N) * (double)K > 2.5e8);
+    }
+    // few FMAs and one result a thread: one wave of the other kernels is as
+    // short as a launch (2.1 us)
+    if (M > 1 && M < 4 && !cplx && !beta && npt == 1 && fma <= 1.5e5) return false;
     if (per_row < 64.0) {
         if (slow_split && M >= 3) return fma <= 1e6 || cheaper();
         if (M >= 12) return fma <= 8e6 || cheaper();
@@ -512,7 +524,8 @@ tsm_status choose(tsm_kind kind, int dtype, int M, int N, int64_t K, int* varian
         }
     }
     if (g <= 0) g = default_grid((*t)[v], M, N, K);
-    if (kind != TSM_KIND_TSMTTSM && distance != 0 && mm_preferred((*t)[v].info, g, distance, dtype, M, N, K)) {
+    if (kind != TSM_KIND_TSMTTSM && distance != 0 &&
+        mm_preferred((*t)[v].info, g, distance, dtype, M, N, K, kind == TSM_KIND_TSMM_BETA)) {
         static const int row[2] = {find_named(TSM_KIND_TSMM, "tsmm_r64_row"), find_named(TSM_KIND_TSMM, "tsmm_c64_row")};
         if (row[dtype == TSM_C64] >= 0) {
             v = row[dtype == TSM_C64];

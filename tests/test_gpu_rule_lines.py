@@ -39,3 +39,14 @@ def test_ctas_per_sm_of_the_row_kernel(tsm, cplx, M, N, K, per_sm):
     import torch
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     assert _choice(tsm, tsm.KIND_TSMTTSM, cplx, M, N, K) == (True, per_sm * sms)
+
+
+@pytest.mark.parametrize("beta,M,N,K,row", [
+    (1, 2, 39, 8874093, False), (0, 2, 39, 8874093, True), (1, 2, 45, 184608, True),  # B read as well, from DRAM
+    (0, 2, 23, 200000, False), (0, 2, 23, 2000000, True),                            # one result a thread, from L2
+    (0, 32, 1, 4955571, False), (0, 33, 1, 4955571, True),                           # one column
+    (0, 2, 4, 10800, False), (0, 2, 19, 7000, True)])                               # as short as a launch
+def test_tsmm(tsm, beta, M, N, K, row):
+    kind = tsm.KIND_TSMM_BETA if beta else tsm.KIND_TSMM
+    names = {v["index"]: v["name"] for v in tsm.variants(tsm.KIND_TSMM)}
+    assert names[tsm.choose(kind, 0, M, N, K)[0]].endswith("_row") is row
