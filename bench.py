@@ -431,7 +431,7 @@ def run_ours(args, bw, bw_src):
             out = torch.zeros((M, N), dtype=A.dtype, device=dev)
             var, grid = tsm.choose(tsm.KIND_TSMTTSM, kdt[cplx], M, N, K)
             fn = (lambda A=A, B=B, out=out, op=("C" if cplx else "T"): tsm.tsmttsm(A, B, out, op=op))
-            launches = lib.tsm_tsmttsm_kernels_per_call(kdt[cplx], M, N, grid)
+            launches = lib.tsm_tsmttsm_variant_kernels(var, kdt[cplx], M, N, grid)
         else:
             Cm = _mat(flatC, M, N, cplx)
             out = _mat(Bout, K, N, cplx)

@@ -167,8 +167,11 @@ int tsm_variant_supports(tsm_kind kind, int index, tsm_dtype dtype, int M, int N
  * CTAs: 1, or 2 when the CTA partials (grid * M * N doubles, twice that for
  * complex) are many enough that a separate final kernel sums them (Sec. 3.2
  * reduction, second pass).  The row variants (tsmttsm_*_row, which short
- * products take) always make 2.  -1 for a shape outside [1, 64] or grid < 1. */
+ * products take) always make 2: tsm_tsmttsm_variant_kernels answers for a
+ * variant (as tsm_choose returns it).  -1 for a shape outside [1, 64], grid < 1
+ * or a variant that does not support the shape. */
 int tsm_tsmttsm_kernels_per_call(tsm_dtype dtype, int M, int N, int grid);
+int tsm_tsmttsm_variant_kernels(int variant, tsm_dtype dtype, int M, int N, int grid);
 
 /*
  * As tsm_tsmttsm / tsm_tsmm but with an explicit variant and grid size

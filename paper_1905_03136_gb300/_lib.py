@@ -63,6 +63,7 @@ SIGNATURES = {
     "tsm_variant_get": (i32, [i32, i32, ctypes.POINTER(VariantInfo)]),
     "tsm_variant_supports": (i32, [i32, i32, i32, i32, i32]),
     "tsm_tsmttsm_kernels_per_call": (i32, [i32, i32, i32, i32]),
+    "tsm_tsmttsm_variant_kernels": (i32, [i32, i32, i32, i32, i32]),
     "tsm_choose": (i32, [i32, i32, i32, i32, i64, ctypes.POINTER(i32), ctypes.POINTER(i32)]),
     "tsm_fill_random": (i32, [vp, i32, i64, i64, i64, u64, i32, vp]),
     "tsm_tune": (i32, [i32, i32, i32, i32, i64, vp, i64, vp, i64, vp, i64, i32,

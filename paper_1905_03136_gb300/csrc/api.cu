@@ -621,7 +621,7 @@ tsm_status run_tsmttsm(tsm_op opA, tsm_dtype dtype, int M, int N, int64_t K, con
     a.conj = (cplx && opA == TSM_OP_C) ? 1 : 0;
     a.ws = ws->partials;
     a.ticket = ws->tickets;
-    a.final_pass = var.final_pass || tsm_tsmttsm_kernels_per_call(dtype, M, N, g) == 2 ? 1 : 0;
+    a.final_pass = tsm_tsmttsm_variant_kernels(v, dtype, M, N, g) == 2 ? 1 : 0;
     const Range in[2] = {operand_range(A, K, lda, M, cplx), operand_range(B, K, ldb, N, cplx)};
     std::lock_guard<std::mutex> lock(pdl_mutex());
     a.early = pdl_early(stream, in, 2);
@@ -791,6 +791,12 @@ tsm_status tsm_variant_shape(tsm_kind kind, int index, tsm_dtype dtype, int M, i
 int tsm_tsmttsm_kernels_per_call(tsm_dtype dtype, int M, int N, int grid) {
     if (M < 1 || N < 1 || M > 64 || N > 64 || grid < 1 || (dtype != TSM_R64 && dtype != TSM_C64)) return -1;
     return (int64_t)grid * M * N * (dtype == TSM_C64 ? 2 : 1) > kFinalThreshold ? 2 : 1;
+}
+
+int tsm_tsmttsm_variant_kernels(int variant, tsm_dtype dtype, int M, int N, int grid) {
+    const int n = tsm_tsmttsm_kernels_per_call(dtype, M, N, grid);
+    if (n < 0 || !supports(TSM_KIND_TSMTTSM, variant, dtype, M, N)) return -1;
+    return variant_at(TSM_KIND_TSMTTSM, variant)->final_pass ? 2 : n;
 }
 
 int tsm_variant_supports(tsm_kind kind, int index, tsm_dtype dtype, int M, int N) {

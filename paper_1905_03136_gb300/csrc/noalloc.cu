@@ -108,7 +108,7 @@ extern "C" tsm_status tsm_tsmttsm_noalloc(tsm_op opA, tsm_dtype dtype, int M, in
     a.ws = static_cast<double*>(scratch);
     a.ticket = ticket;
     // many partials: a separate final kernel sums them (it allocates nothing)
-    a.final_pass = var->final_pass || tsm_tsmttsm_kernels_per_call(dtype, M, N, grid) == 2 ? 1 : 0;
+    a.final_pass = tsm_tsmttsm_variant_kernels(variant, dtype, M, N, grid) == 2 ? 1 : 0;
     // the ticket reset above already orders this launch after the previous
     // one; the record lets the next product know what this one writes
     std::lock_guard<std::mutex> lock(pdl_mutex());
