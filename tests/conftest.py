@@ -28,3 +28,16 @@ def pytest_collection_modifyitems(config, items):
     for item in items:
         if "gpu" in item.keywords:
             item.add_marker(skip)
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _tuning_table_as_shipped():
+    """Entries that a module's tests add to the process-wide tuning table do
+    not reach the next module's."""
+    yield
+    package = sys.modules.get("paper_1905_03136_gb300._lib")
+    if package is not None and package._lib is not None:
+        path = os.environ.get("TSM_TUNE_FILE") or package.DEFAULT_TABLE
+        if os.path.exists(path):
+            package._lib.tsm_clear_tuning()
+            package._lib.tsm_load_tuning(path.encode())
