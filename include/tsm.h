@@ -27,6 +27,11 @@
  * errors and launch errors are reported synchronously.  Results are
  * bitwise reproducible from run to run for a fixed kernel variant, device and
  * problem (the reductions have a fixed order; no floating-point atomics).
+ * Consecutive products on a stream overlap: one may start, and read its
+ * inputs, while the product before it finishes.  Inputs that other code's
+ * kernels write are waited for, unless such a kernel lets its dependents start
+ * (programmatic dependent launch) before it has written them: then put an
+ * ordinary launch in between, or set TSM_PDL=0 in the environment.
  *
  * Error behaviour.  Every entry point validates all arguments before
  * enqueueing anything; on an error nothing is launched and the outputs are

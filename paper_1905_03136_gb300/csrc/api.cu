@@ -48,17 +48,31 @@ std::map<std::pair<int, cudaStream_t>, Workspace*> g_ws;
 
 }  // namespace
 
-// Clears device memory before returning.  A memset on the legacy stream alone
-// would neither wait for nor hold back work on a non-blocking stream, and one
-// on the caller's stream would become part of a graph being captured there.
+// One non-blocking stream per device, made on first use and kept until exit,
+// for set-up that is waited for.  On the legacy stream it would neither wait
+// for nor hold back work on a non-blocking stream, and on the caller's it
+// would become part of a graph being captured there.
+cudaError_t setup_stream(cudaStream_t* out) {
+    static std::mutex mu;
+    static cudaStream_t streams[64] = {nullptr};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lock(mu);
+    if (!streams[dev] && (e = cudaStreamCreateWithFlags(&streams[dev], cudaStreamNonBlocking)) != cudaSuccess) {
+        streams[dev] = nullptr;
+        return e;
+    }
+    *out = streams[dev];
+    return cudaSuccess;
+}
+
 cudaError_t zero_now(void* p, size_t bytes) {
     cudaStream_t s = nullptr;
-    cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(p, 0, bytes, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaStreamDestroy(s);
-    return e;
+    cudaError_t e = setup_stream(&s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(p, 0, bytes, s);
+    return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
 }
 
 tsm_status workspace_get(cudaStream_t stream, size_t partial_bytes, int tickets, Workspace** out) {

@@ -479,14 +479,11 @@ tsm_status tsm_mlp_create(int in_dim, int hidden, int max_batch, uint64_t seed, 
     for (int i = 0; i < hidden; ++i) h[o.w3 + i] = uni(1.0f / sqrtf((float)hidden));
     // in place before this returns, whatever stream the model is used on
     cudaStream_t cs = nullptr;
-    ok = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess;
-    if (ok) {
-        ok = cudaMemcpyAsync(m->params, h.data(), pb, cudaMemcpyHostToDevice, cs) == cudaSuccess &&
-             cudaMemsetAsync(m->grads, 0, pb, cs) == cudaSuccess && cudaMemsetAsync(m->m, 0, pb, cs) == cudaSuccess &&
-             cudaMemsetAsync(m->v, 0, pb, cs) == cudaSuccess;
-        ok = cudaStreamSynchronize(cs) == cudaSuccess && ok;
-        cudaStreamDestroy(cs);
-    }
+    ok = setup_stream(&cs) == cudaSuccess &&
+         cudaMemcpyAsync(m->params, h.data(), pb, cudaMemcpyHostToDevice, cs) == cudaSuccess &&
+         cudaMemsetAsync(m->grads, 0, pb, cs) == cudaSuccess && cudaMemsetAsync(m->m, 0, pb, cs) == cudaSuccess &&
+         cudaMemsetAsync(m->v, 0, pb, cs) == cudaSuccess;
+    if (cs) ok = cudaStreamSynchronize(cs) == cudaSuccess && ok;
     if (!ok) {
         tsm_mlp_destroy(m);
         return TSM_ERR_LAUNCH;

@@ -179,7 +179,9 @@ struct Workspace {
 };
 tsm_status workspace_get(cudaStream_t stream, size_t partial_bytes, int tickets, Workspace** out);
 
-// Clears device memory before returning (api.cu).
+// The device's stream for set-up that is waited for, and device memory cleared
+// there before returning (api.cu).
+cudaError_t setup_stream(cudaStream_t* out);
 cudaError_t zero_now(void* p, size_t bytes);
 
 // The Gram-Schmidt step as one cooperative kernel (gs_fused.cu), and the
