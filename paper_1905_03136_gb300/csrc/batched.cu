@@ -645,6 +645,8 @@ RowCost row_cost(const Inst& in) {
 // of 2^14 .. 2^18, 0.95, 0.95, 1.06 ms for 64 of 2^10 .. 2^12.  Equal items of
 // at least 4096 rows, the split before this one, took 1231, 29.4 and 22.4 ms:
 // a 4096-row item of a complex 64 x 64 product alone takes 16 ms on one CTA.
+// Larger items are longer chains: error against 64 bits of the 32 products
+// 3.0e-15, 2.8e-15 with equal ones.
 struct Tier {
     double part, share;
 };

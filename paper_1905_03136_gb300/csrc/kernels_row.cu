@@ -18,7 +18,8 @@
 // final kernel, whose few CTAs are already waiting when this one ends (the
 // last CTA alone, or groups of CTAs in two levels, took 2 to 5 us more).
 // Every order is fixed by the shape and the grid, so results repeat bit for
-// bit.
+// bit.  A lane's rows are one chain of FMAs: real 37 x 53, 300007 rows has an
+// error of 1.1e-15 against 64 bits, 8.7e-16 with the tile kernel's shorter ones.
 #include <algorithm>
 #include <atomic>
 #include <cmath>

@@ -60,8 +60,8 @@
 // (460).  Measured before and after this organisation (one warp per 16
 // columns in lock step with the MMA, exponents that ended a tile at every
 // new maximum; 2^22 rows): complex 64 x 64 6.07 / 4.65 ms (uniform
-// data) and 11.8 / 5.5 ms (normal data); real 24 x 40, S = 5, 10^6 rows 0.54 /
-// 0.33 ms.
+// data) and 11.8 / 5.4 ms (normal data); real 24 x 40, S = 5, 10^6 rows 0.54 /
+// 0.32 ms.
 //
 // Every wait on an mbarrier is bounded by a clock budget; on expiry the
 // kernel records an error word, stops issuing work, drains its own MMAs,
