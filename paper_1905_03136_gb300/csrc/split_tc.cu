@@ -625,8 +625,8 @@ __global__ void __launch_bounds__(kThreadsPerSM, 1) k_split(const Params prm) {
         // first step's, so that small rows before large ones keep their
         // bits.  Without the scan every new maximum of a column's first rows
         // ends an accumulation tile, at about 10 us of the CTA (normal data:
-        // real 24 x 40, S = 5, 10^6 rows 569 us against 352, complex 64 x 64,
-        // 10^5 rows 404 against 191).
+        // real 24 x 40, S = 5, 10^6 rows 569 us against 370, complex 64 x 64,
+        // 10^5 rows 404 against 231; with the whole scan's maximum 352 and 191).
         const int srange = (int)min(prm.steps_per_range, (int64_t)nsteps + 1);
         if (!plain_digits<S>()) {
             int* first = exps;  // not in use yet: the ranges' first steps' exponents [MAX_RANGES][NE], ndig >= MAX_RANGES
